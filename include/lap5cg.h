@@ -150,10 +150,15 @@ typedef struct {
                                (bulk asynchronous copies): 0 = automatic (on when the warp
                                units are at least 8 rows tall),
                                3..8 = that many, < 0 = no ring (rows loaded into registers) */
-  int32_t resident;         /* F64 / F32 solves of grids that fit in the shared memory of one
-                               thread-block cluster (about 250 x 250 binary64): 0 = solve them
-                               there (default, when ring_slots == 0 and rr_period == 0),
-                               < 0 = always use the streaming kernels */
+  int32_t resident;         /* 0 (default): F64, F32 classic and IR_F32 solves whose vectors fit in
+                               the registers and shared memory of the chip (about 1060^2
+                               binary64, 680^2 for NewCG, 1470^2 binary32 and IR_F32) are solved
+                               there, unless an option that shapes other kernels is set (ctas,
+                               warps_per_cta, min_rows, ring_slots, lane_vec, store_z, team_ctas,
+                               rr_period, reproducible, stabilized); F64 / F32 grids left that fit
+                               in the shared memory of one thread-block cluster (about 250 x 250
+                               binary64) are solved there when ring_slots == 0 and
+                               rr_period == 0.  < 0: always the streaming kernels */
   int32_t lane_vec;         /* columns each lane owns in its warp's strip.
                                Binary32 passes (F32 classic; the inner passes of IR_F32 /
                                IR_BF16PR): 4 or 8; 0 = automatic (8 when nx >= 1024 and the
@@ -251,13 +256,13 @@ LAP5CG_API size_t cg_batched_workspace_size(int count, const int* nx, const int*
                                  int variant, int precision);
 
 /*
- * Solve count independent systems A_k x_k = b_k of different shapes in one
- * persistent launch.  Each instance is solved by a team of CTAs forming one
- * thread-block cluster (cluster barrier, reductions through distributed shared
- * memory); teams take instances from a device-side queue ordered by estimated
- * work, largest first, so an instance that has converged stops and its team
- * takes the next one (per-instance convergence masking).  Per instance the
- * arithmetic is that of cg_solve (Algorithm 1 / 2, same precisions).
+ * Solve count independent systems A_k x_k = b_k of different shapes in a few
+ * persistent launches.  Each instance is solved by a team of CTAs -- SMs that hold
+ * its vectors in registers and shared memory where they fit (opts.resident), else
+ * one thread-block cluster; teams take instances from a device-side queue ordered
+ * by estimated work, largest first, so an instance that has converged stops and
+ * its team takes the next one (per-instance convergence masking).  Per instance
+ * the arithmetic is that of cg_solve (Algorithm 1 / 2, same precisions).
  *   count     : 1 .. LAP5CG_MAX_BATCH.
  *   nx, ny, ld: host arrays of count shapes; every ld must be a multiple of
  *               the lane vector width (2 for F64, 4 otherwise) and every b, x

@@ -271,7 +271,9 @@ int cg_solve(int nx, int ny, int ld, const void* b, void* x, double tol, int max
     }
     int rc;
     bool done = false;
-    rc = try_small(p, st, &done);  // small grids: one cluster, shared-memory resident
+    rc = try_resident(p, st, &done);  // state vectors in the SMs' registers and shared memory
+    if (rc != LAP5CG_OK) return rc;
+    if (!done) rc = try_small(p, st, &done);  // small grids: one cluster, shared-memory resident
     if (rc != LAP5CG_OK) return rc;
     if (!done) {
       switch (precision) {

@@ -18,14 +18,6 @@
 
 namespace lap5 {
 
-struct BatchEntry {
-  const void* b;
-  void* x;
-  long long ws_off;  // byte offset of this instance's vectors in the workspace
-  int nx, ny, ld;
-  int idx;           // position in the caller's arrays (info slot)
-};
-
 struct BatchCtl {
   unsigned int next;  // queue head
   int pad[63];
@@ -253,6 +245,23 @@ size_t batched_ws(int count, const int* nx, const int* ny, const int* ld, int va
   return s;
 }
 
+int fill_batch_table(BatchEntry* dst, const BatchEntry* src, int n, cudaStream_t st) {
+  for (int first = 0; first < n; first += kFillChunk) {
+    FillArgs fa;
+    fa.dst = dst;
+    fa.first = first;
+    fa.n = std::min(kFillChunk, n - first);
+    for (int k = 0; k < fa.n; ++k) fa.e[k] = src[first + k];
+    k_fill_table<<<1, kFillChunk, 0, st>>>(fa);
+    if (cudaGetLastError() != cudaSuccess) return LAP5CG_ERR_CUDA;
+  }
+  return LAP5CG_OK;
+}
+
+size_t batched_instance_bytes(int nx, int ny, int ld, int variant, int precision) {
+  return instance_bytes(kind_of(variant, precision), nx, ny, ld);
+}
+
 int solve_batched(int count, const int* nx, const int* ny, const int* ld, const void* const* b, void* const* x,
                   double tol, int maxit, int variant, int precision, void* workspace, size_t ws_bytes,
                   lap5cg_info* info, const lap5cg_opts& o, cudaStream_t st) {
@@ -274,11 +283,25 @@ int solve_batched(int count, const int* nx, const int* ny, const int* ld, const 
     if (b0 < x0 + bytes && x0 < b0 + bytes) return LAP5CG_ERR_INVALID_ARG;
     order[k] = k;
   }
-  // instances that fit in one cluster's shared memory (F64 / F32): the
-  // cluster-resident kernel, one cluster an instance, launched first
+  unsigned char* ws = static_cast<unsigned char*>(workspace);
+  BatchCtl* bctl = reinterpret_cast<BatchCtl*>(ws);
+  BatchEntry* dtab = reinterpret_cast<BatchEntry*>(ws + kAlign);
+  int* errs = reinterpret_cast<int*>(ws + kAlign + align_up((size_t)count * sizeof(BatchEntry), kAlign));
+  size_t off = kAlign + table_bytes(count);
+  if (cudaMemsetAsync(errs, 0, (size_t)count * sizeof(int), st) != cudaSuccess) return LAP5CG_ERR_CUDA;  // caller order
+  // instances that fit on a team of SMs (F64, F32 classic, IR_F32): the
+  // chip-resident kernels
   std::vector<char> taken;
-  int rc = small_batched(count, nx, ny, ld, b, x, tol, maxit, variant, precision, info, o, st, taken);
+  int rc = resident_batched(count, nx, ny, ld, b, x, tol, maxit, variant, precision, ws, ws_bytes, dtab, off, errs,
+                            info, o, st, taken, &off);
   if (rc != LAP5CG_OK) return rc;
+  const int ntab = (int)std::count(taken.begin(), taken.end(), (char)1);  // table entries in use
+  // of the others, those that fit in one cluster's shared memory (F64 / F32): the
+  // cluster-resident kernel, one cluster an instance
+  if (ntab < count) {
+    rc = small_batched(count, nx, ny, ld, b, x, tol, maxit, variant, precision, info, o, st, taken);
+    if (rc != LAP5CG_OK) return rc;
+  }
   order.erase(std::remove_if(order.begin(), order.end(), [&](int k) { return taken[k] != 0; }), order.end());
   const int nbig = (int)order.size();
   if (nbig == 0) return LAP5CG_OK;
@@ -287,12 +310,7 @@ int solve_batched(int count, const int* nx, const int* ny, const int* ld, const 
     const double wi = (double)nx[i] * ny[i] * (nx[i] + ny[i]), wj = (double)nx[j] * ny[j] * (nx[j] + ny[j]);
     return wi > wj;
   });
-  unsigned char* ws = static_cast<unsigned char*>(workspace);
-  BatchCtl* bctl = reinterpret_cast<BatchCtl*>(ws);
-  BatchEntry* dtab = reinterpret_cast<BatchEntry*>(ws + kAlign);
-  int* errs = reinterpret_cast<int*>(ws + kAlign + align_up((size_t)count * sizeof(BatchEntry), kAlign));
-  const size_t inst0 = kAlign + table_bytes(count);
-  size_t off = inst0;
+  dtab += ntab;
   tab.resize(nbig);
   for (int k = 0; k < nbig; ++k) {
     const int i = order[k];
@@ -305,17 +323,9 @@ int solve_batched(int count, const int* nx, const int* ny, const int* ld, const 
     tab[k].idx = i;
     off += instance_bytes(kind, nx[i], ny[i], ld[i]);
   }
-  for (int first = 0; first < nbig; first += kFillChunk) {
-    FillArgs fa;
-    fa.dst = dtab;
-    fa.first = first;
-    fa.n = std::min(kFillChunk, nbig - first);
-    for (int k = 0; k < fa.n; ++k) fa.e[k] = tab[first + k];
-    k_fill_table<<<1, kFillChunk, 0, st>>>(fa);
-    if (cudaGetLastError() != cudaSuccess) return LAP5CG_ERR_CUDA;
-  }
+  rc = fill_batch_table(dtab, tab.data(), nbig, st);
+  if (rc != LAP5CG_OK) return rc;
   if (cudaMemsetAsync(bctl, 0, sizeof(BatchCtl), st) != cudaSuccess) return LAP5CG_ERR_CUDA;
-  if (cudaMemsetAsync(errs, 0, (size_t)count * sizeof(int), st) != cudaSuccess) return LAP5CG_ERR_CUDA;  // caller order
 
   int wpc = o.warps_per_cta > 0 ? o.warps_per_cta : 8;  // batched teams measured best with 8
   if (wpc > 16) wpc = 16;

@@ -45,10 +45,35 @@ size_t ws_bytes_f32(int nx, int ny, int ldw, int variant);
 size_t ws_bytes_ir(int nx, int ny, int variant, int precision);
 size_t ws_bytes_mg(int nx, int ny, int ldw, int variant, int precision);
 
+// One instance of a batched solve, as the device-side queue's table holds it.
+struct BatchEntry {
+  const void* b;
+  void* x;
+  long long ws_off;  // byte offset of this instance's memory in the workspace
+  int nx, ny, ld;
+  int idx;           // position in the caller's arrays (info slot)
+};
+int fill_batch_table(BatchEntry* dst, const BatchEntry* src, int n, cudaStream_t st);
+// Workspace bytes of one instance's state vectors.
+size_t batched_instance_bytes(int nx, int ny, int ld, int variant, int precision);
+
+// Batched solves: the instances whose state fits on a team of SMs are solved by
+// the chip-resident kernels; taken[k] is set for them (count entries).  dtab:
+// device table of count entries; their memory starts at first_off of the
+// workspace and ends at *end_off.
+int resident_batched(int count, const int* nx, const int* ny, const int* ld, const void* const* b, void* const* x,
+                     double tol, int maxit, int variant, int precision, unsigned char* ws, size_t ws_bytes,
+                     BatchEntry* dtab, size_t first_off, int* errs, lap5cg_info* info, const lap5cg_opts& o,
+                     cudaStream_t st, std::vector<char>& taken, size_t* end_off);
+
 size_t batched_ws(int count, const int* nx, const int* ny, const int* ld, int variant, int precision);
 int solve_batched(int count, const int* nx, const int* ny, const int* ld, const void* const* b, void* const* x,
                   double tol, int maxit, int variant, int precision, void* workspace, size_t ws_bytes,
                   lap5cg_info* info, const lap5cg_opts& o, cudaStream_t st);
+
+// Chip-resident solve (F64, F32 classic, IR_F32): *used = false when the state
+// does not fit on the chip or the options ask for other kernels.
+int try_resident(const SolvePlan& p, cudaStream_t st, bool* used);
 
 // Cluster-resident solve of a small grid (F64 / F32): *used = false when the
 // grid does not fit or the options ask for the streaming kernels.

@@ -655,7 +655,7 @@ static int small_batched_t(int count, const int* nx, const int* ny, const int* l
   std::vector<SmallArgs<T>> args;
   size_t smem_max = 0;
   for (int k = 0; k < count; ++k) {
-    if (ny[k] < C) continue;
+    if (taken[k] || ny[k] < C) continue;
     int R, ldp;
     const size_t smem = small_smem<T>(nx[k], ny[k], variant, C, &R, &ldp);
     if (smem + sizeof(double) * kRedDoubles + 1024 > (size_t)dp.max_smem_optin) continue;
@@ -716,7 +716,7 @@ static int small_batched_t(int count, const int* nx, const int* ny, const int* l
 int small_batched(int count, const int* nx, const int* ny, const int* ld, const void* const* b, void* const* x,
                   double tol, int maxit, int variant, int precision, lap5cg_info* info, const lap5cg_opts& o,
                   cudaStream_t st, std::vector<char>& taken) {
-  taken.assign(count, 0);
+  taken.resize(count, 0);
   if (precision == LAP5CG_PREC_F64)
     return small_batched_t<double>(count, nx, ny, ld, b, x, tol, maxit, variant, info, o, st, taken);
   if (precision == LAP5CG_PREC_F32)
