@@ -161,19 +161,39 @@ _DT = {torch.float64: DT_F64, torch.float32: DT_F32, torch.bfloat16: DT_BF16}
 def lap5_apply(x: torch.Tensor, nx: int = None, out: torch.Tensor = None, stream=None) -> torch.Tensor:
     """y = A x (Sec. II-B mask, zero Dirichlet boundary) for a (ny, ld) grid."""
     _check_grid(x, "x")
-    if x.dim() != 2 or x.dtype not in _DT:
+    dt = _DT.get(x.dtype)
+    if x.dim() != 2 or dt is None:
         raise ValueError("x must be a 2D float64/float32/bfloat16 tensor")
     ny, ld = x.shape
     nx = ld if nx is None else int(nx)
     if out is not None:
         _check_like(out, x, "out", "x")
-    y = torch.zeros_like(x) if out is None else out
-    with torch.cuda.device(x.device):
-        rc = lib().lap5_apply(nx, ny, ld, _DT[x.dtype], ctypes.c_void_p(x.data_ptr()),
-                              ctypes.c_void_p(y.data_ptr()), _stream(stream, x.device))
+        y = out
+    else:
+        # the kernel writes every column below nx: only padding is cleared (clearing
+        # all of y first took 35 of 88 us at 8192^2 bf16)
+        y = torch.empty_like(x)
+        if 0 < nx < ld:
+            y[:, nx:].zero_()
+    device = x.device
+    if device.index == torch.cuda.current_device():
+        rc = _apply(nx, ny, ld, dt, x, y, stream, device)
+    else:
+        with torch.cuda.device(device):
+            rc = _apply(nx, ny, ld, dt, x, y, stream, device)
     if rc != OK:
         raise Lap5cgError(rc, "lap5_apply")
     return y
+
+
+# the current stream's handle without building a Stream object (2 us of a 4 us call)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+    lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
+def _apply(nx, ny, ld, dt, x, y, stream, device):
+    handle = _raw_stream(device.index) if stream is None else stream.cuda_stream
+    return (_lib or lib()).lap5_apply(nx, ny, ld, dt, x.data_ptr(), y.data_ptr(), handle)
 
 
 def workspace_size(nx, ny, ld, variant="classic", precision="f64", nrhs=1) -> int:
