@@ -18,6 +18,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "fixstencil.cuh"
 #include "ring.cuh"
 #include "repro.cuh"
 
@@ -167,6 +168,9 @@ __device__ void classic_solve(const ClassicArgs<T>& a, Team& tm, double* red, un
   using M = typename Math<T>::type;
   // EX: reproducible (exact) dot products
   using Acc = typename std::conditional<EX, AccExact, typename AccOf<M>::type>::type;
+  // binary64 through the ring: the stencil in fixed point (the reproducible mode
+  // fixes the order of the FP64 sum)
+  constexpr bool FIX = sizeof(M) == 8 && R && !EX;
   const SolveCommon& c = a.c;
   Walker wk;
   wk.init(tm.rank(), tm.size());
@@ -258,15 +262,23 @@ __device__ void classic_solve(const ClassicArgs<T>& a, Team& tm, double* red, un
               }
               f.hr = f.hl;
             };
-            auto finish = [&](int j, const unsigned char*, const FRow<V, M>& S, const FRow<V, M>& C,
-                              const FRow<V, M>& N) {
-              M ap[V];
-              stencil_row<V>(S, C, N, wk.lane, ap);
-              store_row<V>(pnew, j, xl, c.nx, C.f);
+            auto row = [&](int j, const M (&p)[V], const M (&ap)[V]) {
+              store_row<V>(pnew, j, xl, c.nx, p);
               if (a.store_z) store_row<V>(a.z, j, xl, c.nx, ap);
-              acc_dot<V>(acc, j, C.f, ap, nval);
+              acc_dot<V>(acc, j, p, ap, nval);
             };
-            march_ring<V, M>(ring, c.ny, xs, y0, y1, wk.rev(), vv, off, field, finish);
+            if constexpr (FIX) {
+              auto finish = [&](int j, const unsigned char*, const M (&p)[V], const M (&ap)[V]) { row(j, p, ap); };
+              march_ring_fix<V>(ring, c.ny, wk.lane, xs, y0, y1, wk.rev(), vv, off, field, finish);
+            } else {
+              auto finish = [&](int j, const unsigned char*, const FRow<V, M>& S, const FRow<V, M>& C,
+                                const FRow<V, M>& N) {
+                M ap[V];
+                stencil_row<V>(S, C, N, wk.lane, ap);
+                row(j, C.f, ap);
+              };
+              march_ring<V, M>(ring, c.ny, xs, y0, y1, wk.rev(), vv, off, field, finish);
+            }
           }
         } else
         for (int u = wk.gw; u < c.un.nunits; u += wk.nw) {
@@ -585,6 +597,9 @@ __device__ void newcg_solve(const NewcgArgs<T>& a, Team& tm, double* red, unsign
   using M = typename Math<T>::type;
   // EX: reproducible (exact) dot products
   using Acc = typename std::conditional<EX, AccExact, typename AccOf<M>::type>::type;
+  // binary64 through the ring: the stencil in fixed point (the reproducible mode
+  // fixes the order of the FP64 sum)
+  constexpr bool FIX = sizeof(M) == 8 && R && !EX;
   const SolveCommon& c = a.c;
   Walker wk;
   wk.init(tm.rank(), tm.size());
@@ -660,10 +675,8 @@ __device__ void newcg_solve(const NewcgArgs<T>& a, Team& tm, double* red, unsign
             f.hl = ring_halo<V, T, M>(sl, off[0], wk.lane, xs, c.nx);
             f.hr = f.hl;
           };
-          auto finish = [&](int j, const unsigned char* sl, const FRow<V, M>& S, const FRow<V, M>& C,
-                            const FRow<V, M>& N) {
-            M nv[V], zv[V], qv[V], pv[V], xv[V], rv[V], wv[V];
-            stencil_row<V>(S, C, N, wk.lane, nv);  // n = A w
+          auto row = [&](int j, const unsigned char* sl, const M (&w0)[V], const M (&nv)[V]) {  // n = A w
+            M zv[V], qv[V], pv[V], xv[V], rv[V], wv[V];
             ring_lane<V, T>(sl, off[4], false, wk.lane, xl, c.nx, xv);
             ring_lane<V, T>(sl, off[5], false, wk.lane, xl, c.nx, rv);
             if (!first) {
@@ -675,16 +688,16 @@ __device__ void newcg_solve(const NewcgArgs<T>& a, Team& tm, double* red, unsign
             for (int k = 0; k < V; ++k) {
               if (first) {
                 zv[k] = nv[k];
-                qv[k] = C.f[k];
+                qv[k] = w0[k];
                 pv[k] = rv[k];
               } else {
                 zv[k] = fmx(bm, zv[k], nv[k]);
-                qv[k] = fmx(bm, qv[k], C.f[k]);
+                qv[k] = fmx(bm, qv[k], w0[k]);
                 pv[k] = fmx(bm, pv[k], rv[k]);
               }
               xv[k] = fmx(am, pv[k], xv[k]);
               rv[k] = fmx(-am, qv[k], rv[k]);
-              wv[k] = fmx(-am, zv[k], C.f[k]);
+              wv[k] = fmx(-am, zv[k], w0[k]);
             }
             acc_dot<V>(ag, j, rv, rv, nval);
             acc_dot<V>(ad, j, wv, rv, nval);
@@ -699,7 +712,17 @@ __device__ void newcg_solve(const NewcgArgs<T>& a, Team& tm, double* red, unsign
             store_row<V>(a.r, j, xl, c.nx, rv);
             store_row<V>(wn, j, xl, c.nx, wv);
           };
-          march_ring<V, M>(ring, c.ny, xs, y0, y1, wk.rev(), vv, off, field, finish);
+          if constexpr (FIX) {
+            march_ring_fix<V>(ring, c.ny, wk.lane, xs, y0, y1, wk.rev(), vv, off, field, row);
+          } else {
+            auto finish = [&](int j, const unsigned char* sl, const FRow<V, M>& S, const FRow<V, M>& C,
+                              const FRow<V, M>& N) {
+              M nv[V];
+              stencil_row<V>(S, C, N, wk.lane, nv);
+              row(j, sl, C.f, nv);
+            };
+            march_ring<V, M>(ring, c.ny, xs, y0, y1, wk.rev(), vv, off, field, finish);
+          }
         }
       } else
       for (int u = wk.gw; u < c.un.nunits; u += wk.nw) {
