@@ -33,6 +33,20 @@ int warps_of(const lap5cg_opts& o) {
   return wpc > 16 ? 16 : wpc;
 }
 
+static int ring_warp_bytes(int S, int slot_bytes) { return (int)align_up(128 + (size_t)S * slot_bytes, 128); }
+
+lap5cg_opts with_warps(const lap5cg_opts& o, int slot_bytes) {
+  lap5cg_opts r = o;
+  r.warps_per_cta = warps_of(o);
+  DevProps dp;
+  if (o.warps_per_cta > 0 || o.ring_slots <= 0 || dev_props(&dp) != LAP5CG_OK) return r;
+  const int S = o.ring_slots < 3 ? 3 : (o.ring_slots > kRingMaxSlots ? kRingMaxSlots : o.ring_slots);
+  while (r.warps_per_cta > 4 &&
+         (size_t)r.warps_per_cta * ring_warp_bytes(S, slot_bytes) + 4096 > (size_t)dp.max_smem_optin)
+    r.warps_per_cta /= 2;
+  return r;
+}
+
 int plan_units(const void* func, int nx, int ny, int V, const lap5cg_opts& o, size_t dyn_smem, LaunchCfg* cfg,
                int row_align) {
   DevProps dp;
@@ -78,7 +92,7 @@ int choose_ring(const void* func, int slot_bytes, const lap5cg_opts& o, int wpc,
     if (S > 6) S = 6;
     if (S < 3) return LAP5CG_OK;  // too little room: register march
   }
-  const int warp_bytes = (int)align_up(128 + (size_t)S * slot_bytes, 128);
+  const int warp_bytes = ring_warp_bytes(S, slot_bytes);
   const size_t dyn = (size_t)wpc * warp_bytes;
   DevProps dp;
   int rc = dev_props(&dp);

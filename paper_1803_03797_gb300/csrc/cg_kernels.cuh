@@ -218,7 +218,7 @@ __device__ void classic_solve(const ClassicArgs<T>& a, Team& tm, double* red, un
       const bool upd_x = defer && !first;  // apply iteration k-1's x update in this phase P
       const M ap_prev = (M)alpha_prev;
       // ---------------- phase P ----------------
-      double pap;
+      double pap, al[2];
       {
         Acc acc = make_acc<Acc>(tm, 0, c.ny, wk.rev());
         const M bm = (M)beta;
@@ -327,12 +327,25 @@ __device__ void classic_solve(const ClassicArgs<T>& a, Team& tm, double* red, un
         }
         ++wk.pc;
         double o[1];
-        if (!acc_reduce<1>(tm, {&acc}, o, red)) { aborted = true; goto done; }
+        // alpha, and beside it in lane 1 the reciprocal that the next beta starts from
+        const double gm = gamma;
+        auto post = [gm](const double (&s)[1], double (&e)[2]) {
+          if constexpr (EX) {
+            e[0] = gm / s[0];
+            e[1] = 0.0;
+          } else {
+            const bool l1 = (threadIdx.x & 31) == 1;
+            const double q = (l1 ? 1.0 : gm) / (l1 ? gm : s[0]);
+            e[0] = __shfl_sync(0xffffffffu, q, 0);
+            e[1] = __shfl_sync(0xffffffffu, q, 1);
+          }
+        };
+        if (!acc_reduce<1, 2>(tm, {&acc}, o, al, red, post)) { aborted = true; goto done; }
         pap = o[0];
       }
-      if (!(pap > 0.0) || !isfinite(pap)) { status = LAP5CG_ERR_BREAKDOWN; goto truecheck; }
+      if (!bits_positive(pap) || !bits_finite(pap)) { status = LAP5CG_ERR_BREAKDOWN; goto truecheck; }
       {
-        const double alpha = gamma / pap;
+        const double alpha = al[0];
         const M am = (M)alpha;
         Acc acc = make_acc<Acc>(tm, 0, c.ny, wk.rev());
         if constexpr (R) {
@@ -436,8 +449,13 @@ __device__ void classic_solve(const ClassicArgs<T>& a, Team& tm, double* red, un
           }
         }
         ++wk.pc;
-        double o[1];
-        if (!acc_reduce<1>(tm, {&acc}, o, red)) { aborted = true; goto done; }
+        double o[1], be[1];
+        const double gm = gamma, rg = al[1];
+        auto post = [gm, rg](const double (&s)[1], double (&e)[1]) {
+          if constexpr (EX) e[0] = s[0] / gm;
+          else e[0] = quotient(s[0], gm, rg);
+        };
+        if (!acc_reduce<1, 1>(tm, {&acc}, o, be, red, post)) { aborted = true; goto done; }
         const double gnew = o[0];
         ++iters;
         if (defer) {
@@ -446,11 +464,11 @@ __device__ void classic_solve(const ClassicArgs<T>& a, Team& tm, double* red, un
           plast = pnew;
         }
         if (c.history && tm.rank() == 0 && threadIdx.x == 0) c.history[iters] = sqrt(gnew / bb);
-        if (!isfinite(gnew)) { status = LAP5CG_ERR_NONFINITE; gamma = gnew; goto finalx; }
-        beta = gnew / gamma;
+        if (!bits_finite(gnew)) { status = LAP5CG_ERR_NONFINITE; gamma = gnew; goto finalx; }
+        beta = be[0];
         gamma = gnew;
         cur ^= 1;
-        if (gnew <= thr) { status = LAP5CG_OK; goto finalx; }
+        if (bits_le(gnew, thr)) { status = LAP5CG_OK; goto finalx; }
       }
     }
   }
@@ -608,7 +626,7 @@ __device__ void newcg_solve(const NewcgArgs<T>& a, Team& tm, double* red, unsign
 
   int status = LAP5CG_NOT_CONVERGED, iters = 0;
   double bb = 0.0, gamma = 0.0, delta = 0.0, alpha = 0.0, beta = 0.0, relres_true = nan("");
-  double eps = 0.0, mu = 0.0;  // stabilised form: (r, q_old), (p_old, q_old)
+  double ralpha = 0.0, rgamma = 0.0;  // 1 / alpha, 1 / gamma (plain dot products)
   bool aborted = false;
   int cur = 0;  // current w lives in w[cur]
 
@@ -643,6 +661,8 @@ __device__ void newcg_solve(const NewcgArgs<T>& a, Team& tm, double* red, unsign
     if (!(delta > 0.0) || !isfinite(delta)) { status = LAP5CG_ERR_BREAKDOWN; goto truecheck; }
     alpha = gamma / delta;  // beta = 0
     beta = 0.0;
+    ralpha = delta / gamma;
+    rgamma = 1.0 / gamma;
     for (;;) {
       const bool first = (iters == 0);
       const Grid<T> w = cur ? a.w1 : a.w0;
@@ -776,7 +796,39 @@ __device__ void newcg_solve(const NewcgArgs<T>& a, Team& tm, double* red, unsign
       ++wk.pc;
       ++iters;
       cur ^= 1;
-      double gnew, dnew;
+      // The next iteration's scalars: beta = gamma / gamma_old and Algorithm 2's
+      // alpha = 1 / (delta/gamma - beta/alpha_old), as gamma / (delta - gamma beta /
+      // alpha_old) with 1 / alpha and 1 / gamma (for the iteration after) beside it
+      // in lanes 1 and 2, one division on the way instead of three.  The
+      // stabilised form replaces the denominator by (p, A p) from the current
+      // vectors, in a fixed order.
+      constexpr int NV = ST ? 4 : 2;
+      const double gold = gamma, ra_old = ralpha, rg_old = rgamma, al_old = alpha;
+      double o[NV], ex[4];  // alpha, beta, 1 / alpha, 1 / gamma
+      auto post = [=](const double (&t)[NV], double (&e)[4]) {
+        const double g = t[0], d = t[1];
+        if constexpr (EX) {
+          const double be = g / gold, dn = d / g - be / al_old;
+          e[0] = 1.0 / dn;
+          e[1] = be;
+          e[2] = dn;
+          e[3] = 0.0;
+        } else {
+          const int lane = threadIdx.x & 31;
+          const double be = quotient(g, gold, rg_old);
+          double dn;
+          if constexpr (ST) {
+            dn = __dadd_rn(__dadd_rn(d, __dmul_rn(__dmul_rn(2.0, be), t[2])), __dmul_rn(__dmul_rn(be, be), t[3]));
+          } else {
+            dn = __fma_rn(-g, __dmul_rn(be, ra_old), d);
+          }
+          const double q = (lane == 0 ? g : lane == 1 ? dn : 1.0) / (lane == 0 ? dn : g);
+          e[0] = __shfl_sync(0xffffffffu, q, 0);
+          e[1] = be;
+          e[2] = __shfl_sync(0xffffffffu, q, 1);
+          e[3] = __shfl_sync(0xffffffffu, q, 2);
+        }
+      };
       if (a.rr_period > 0 && iters % a.rr_period == 0) {
         // residual replacement: r = b - A x; w = A r; q = A p; z = A q
         if (!tm.sync(red)) { aborted = true; goto done; }
@@ -790,54 +842,30 @@ __device__ void newcg_solve(const NewcgArgs<T>& a, Team& tm, double* red, unsign
         if constexpr (ST) {  // q = A p with (r, q), (p, q) of the replaced vectors
           Acc ae2{}, amu2{};
           pass_q_from_p<V>(c, wk, a.p, a.q, a.r, ae2, amu2);
-          double o[4];
-          if (!acc_reduce<4>(tm, {&ag2, &ad2, &ae2, &amu2}, o, red)) { aborted = true; goto done; }
-          gnew = o[0];
-          dnew = o[1];
-          eps = o[2];
-          mu = o[3];
+          if (!acc_reduce<4, 4>(tm, {&ag2, &ad2, &ae2, &amu2}, o, ex, red, post)) { aborted = true; goto done; }
         } else {
           pass_apply<V>(c, wk, a.p, a.q);
-          double o[2];
-          if (!acc_reduce<2>(tm, {&ag2, &ad2}, o, red)) { aborted = true; goto done; }
-          gnew = o[0];
-          dnew = o[1];
+          if (!acc_reduce<2, 4>(tm, {&ag2, &ad2}, o, ex, red, post)) { aborted = true; goto done; }
         }
         pass_apply<V>(c, wk, a.q, a.z);
         if (!tm.sync(red)) { aborted = true; goto done; }
       } else {
         if constexpr (ST) {
-          double o[4];
-          if (!acc_reduce<4>(tm, {&ag, &ad, &ae, &amu}, o, red)) { aborted = true; goto done; }
-          gnew = o[0];
-          dnew = o[1];
-          eps = o[2];
-          mu = o[3];
+          if (!acc_reduce<4, 4>(tm, {&ag, &ad, &ae, &amu}, o, ex, red, post)) { aborted = true; goto done; }
         } else {
-          double o[2];
-          if (!acc_reduce<2>(tm, {&ag, &ad}, o, red)) { aborted = true; goto done; }
-          gnew = o[0];
-          dnew = o[1];
+          if (!acc_reduce<2, 4>(tm, {&ag, &ad}, o, ex, red, post)) { aborted = true; goto done; }
         }
       }
-      if (c.history && tm.rank() == 0 && threadIdx.x == 0) c.history[iters] = sqrt(gnew / bb);
-      const double gold = gamma;
-      gamma = gnew;
-      delta = dnew;
-      if (!isfinite(gamma)) { status = LAP5CG_ERR_NONFINITE; goto truecheck; }
-      if (gamma <= thr) { status = LAP5CG_OK; goto truecheck; }
+      gamma = o[0];
+      if (c.history && tm.rank() == 0 && threadIdx.x == 0) c.history[iters] = sqrt(gamma / bb);
+      if (!bits_finite(gamma)) { status = LAP5CG_ERR_NONFINITE; goto truecheck; }
+      if (bits_le(gamma, thr)) { status = LAP5CG_OK; goto truecheck; }
       if (iters >= c.maxit) break;
-      beta = gamma / gold;
-      if constexpr (ST) {  // (p, A p) of p = r + beta p_old from the current vectors, in a fixed order
-        const double pap = __dadd_rn(__dadd_rn(delta, __dmul_rn(__dmul_rn(2.0, beta), eps)),
-                                     __dmul_rn(__dmul_rn(beta, beta), mu));
-        if (!(pap > 0.0) || !isfinite(pap)) { status = LAP5CG_ERR_BREAKDOWN; goto truecheck; }
-        alpha = gamma / pap;
-      } else {
-        const double denom = delta / gamma - beta / alpha;  // de-garbled alpha update
-        if (!(denom > 0.0) || !isfinite(denom)) { status = LAP5CG_ERR_BREAKDOWN; goto truecheck; }
-        alpha = 1.0 / denom;
-      }
+      alpha = ex[0];
+      beta = ex[1];
+      ralpha = ex[2];
+      rgamma = ex[3];
+      if (!bits_positive(ralpha) || !bits_finite(ralpha)) { status = LAP5CG_ERR_BREAKDOWN; goto truecheck; }
     }
   }
 truecheck:

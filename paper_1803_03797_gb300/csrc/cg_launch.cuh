@@ -113,12 +113,14 @@ struct RingOnly {
 // EX: reproducible dot products.  Their units start at multiples of 16 rows
 // and the first of the control block's three exact accumulators starts at zero.
 template <class T, int V, bool EX = false>
-int solve_typed(const SolvePlan& p, cudaStream_t st) {
+int solve_typed(const SolvePlan& plan, cudaStream_t st) {
+  SolvePlan p = plan;
+  p.opts = with_warps(plan.opts, plan.variant == LAP5CG_CLASSIC ? ring_slot_classic(V, (int)sizeof(T))
+                                                                : ring_slot_newcg(V, (int)sizeof(T)));
   const size_t vec = align_up((size_t)p.ny * (size_t)p.ldw * sizeof(T), kAlign);
   unsigned char* base = p.ws + kCtlBytes;
   auto vecp = [&](int k) { return reinterpret_cast<T*>(base + (size_t)k * vec); };
-  const size_t ctl_zero = EX ? offsetof(Ctl, part) : 256;
-  if (cudaMemsetAsync(p.ws, 0, ctl_zero, st) != cudaSuccess) return LAP5CG_ERR_CUDA;
+  if (cudaMemsetAsync(p.ws, 0, kCtlZeroBytes, st) != cudaSuccess) return LAP5CG_ERR_CUDA;
   const int row_align = EX ? kExactRows : 1;
   LaunchCfg cfg;
   if (p.variant == LAP5CG_CLASSIC) {

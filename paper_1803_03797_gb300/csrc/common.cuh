@@ -10,10 +10,12 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <cooperative_groups.h>
+#include <stddef.h>
 #include <stdint.h>
 #include <type_traits>
 
 #include "../../include/lap5cg.h"
+#include "exchange.cuh"
 
 namespace lap5 {
 
@@ -356,6 +358,19 @@ template <class M> struct AccOf;
 template <> struct AccOf<double> { using type = Acc64; };
 template <> struct AccOf<float> { using type = Acc32; };
 
+// A warp's sum of its lanes' accumulators (all lanes).
+__device__ __forceinline__ double warp_sum(const Acc64& a) { return warp_sum(a.s); }
+__device__ __forceinline__ double warp_sum(const Acc32& a) { return warp_sum(a.s, a.c); }
+__device__ __forceinline__ void warp_sum2(const Acc64& a, const Acc64& b, double (&w)[2]) {
+  const double2 t = warp_sum2(a.s, b.s);
+  w[0] = t.x;
+  w[1] = t.y;
+}
+__device__ __forceinline__ void warp_sum2(const Acc32& a, const Acc32& b, double (&w)[2]) {
+  w[0] = warp_sum(a);
+  w[1] = warp_sum(b);
+}
+
 // ---------------------------------------------------------------------------
 // Control block in the workspace (zeroed by the host before each launch).
 // ---------------------------------------------------------------------------
@@ -375,8 +390,13 @@ struct Ctl {
   unsigned long long xacc[3][kExactSlots][kExactLimbs];
   unsigned xbad[3][kExactSlots];
   unsigned xpad[2];
-  double part[2][kMaxCtas][kMaxVals];  // per-CTA partials, double-buffered by barrier parity
+  // per-CTA partials, double-buffered by barrier parity; launches of at most
+  // kMaxPeers CTAs exchange them as messages here (slots of kSlotWords words)
+  double part[2][kMaxCtas][kMaxVals];
 };
+constexpr size_t kMsgBytes = (size_t)2 * kMaxPeers * kSlotWords * 8;
+// bytes of the control block that a launch finds zero
+constexpr size_t kCtlZeroBytes = offsetof(Ctl, part) + kMsgBytes;
 
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
@@ -400,37 +420,114 @@ __device__ __forceinline__ void record_error(Ctl* ctl, int code) {
   atomicExch(&ctl->abort, 1);
 }
 
-// Grid-wide reduction of NV values with a barrier.  Every thread passes its
-// per-thread contributions in v[]; on return every thread of every CTA holds
-// the same totals in out[] (fixed summation order: lanes, warps, then CTA
-// slots 0..G-1), or the function returns false when the solve must stop
-// (abort flag or barrier timeout).  Needs blockDim.x / 32 <= 32 and
-// kMaxVals * 32 doubles of shared scratch (red).
-template <int NV>
-__device__ __forceinline__ bool grid_reduce(Ctl* ctl, unsigned long long& epoch, const double (&v)[NV],
-                                            double (&out)[NV], double* red, long long timeout_ns) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  double t[NV];
+// What a reduction's totals are turned into on one warp (nothing here).
+struct NoScalars {
+  template <int NV, int NE>
+  __device__ void operator()(const double (&)[NV], double (&e)[NE]) const {
 #pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    double s = v[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    t[k] = s;
+    for (int k = 0; k < NE; ++k) e[k] = 0.0;
   }
+};
+
+// Rows of kMaxVals doubles in a kernel's reduction scratch (red).
+enum { RED_WARPS = 0, RED_TOTAL = 32, RED_CLUSTER = 33, RED_POLL = 35, RED_EXTRA = 35 + kPollWarps, RED_ROWS };
+
+// Grid-wide reduction of NV values with a barrier.  w[]: the warp's sums (the same
+// in all its lanes).  On return every thread of every CTA holds the same totals in
+// out[] and in ex[] what post(totals, ex) formed from them; or the function
+// returns false when the solve must stop (abort flag or time limit).  Global writes
+// of every CTA before the call are visible to every CTA after it.
+//
+// post runs on one warp a CTA: an FP64 division is a chain of nine operations, and in
+// each of an SM's 16 warps the four of a NewCG iteration took 4 us.
+//
+// Launches of at most kMaxPeers CTAs (one a SM, the default) exchange the CTA sums
+// as messages (exchange.cuh); larger ones count arrivals at one address and read
+// the partial sums afterwards.
+template <int NV, int NE, class Post>
+__device__ __forceinline__ bool grid_reduce_post(Ctl* ctl, unsigned long long& epoch, const double (&w)[NV],
+                                                 double (&out)[NV], double (&ex)[NE], double* red,
+                                                 long long timeout_ns, Post post) {
+  static_assert(NV <= kMaxVals && NE <= kMaxVals, "scratch rows");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   __shared__ int s_go;
   if (lane == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) red[warp * kMaxVals + k] = t[k];
+    for (int k = 0; k < NV; ++k) red[(RED_WARPS + warp) * kMaxVals + k] = w[k];
   }
+  if (threadIdx.x == 0) s_go = 1;
   __syncthreads();
   const int par = (int)(epoch & 1ull);
-  if (warp == 0) {
+  if ((int)gridDim.x <= kMaxPeers && nwarps >= kPollWarps) {
+    const uint32_t tag = (uint32_t)epoch + 1u;
+    u64* slots = reinterpret_cast<u64*>(&ctl->part[0][0][0]) + (size_t)par * kMaxPeers * kSlotWords;
+    if (warp < NV) {
+      const double s = warp_sum(lane < nwarps ? red[(RED_WARPS + lane) * kMaxVals + warp] : 0.0);
+      if (lane == 0) {
+        __threadfence();
+        ll_send(slots + (size_t)blockIdx.x * kSlotWords + 2 * warp, s, tag);
+      }
+    }
+    const int pw = warp - (nwarps - kPollWarps);
+    if (pw >= 0) {
+      const int c = 32 * pw + lane;
+      double v[NV];
+#pragma unroll
+      for (int k = 0; k < NV; ++k) v[k] = 0.0;
+      // read while the messages travel; a flag set later is seen at the next barrier
+      const int aborted = ld_relaxed_i32(&ctl->abort);
+      unsigned spins = 0;
+      unsigned long long t0 = 0;
+      for (;;) {
+        bool ok = true;
+        if (c < (int)gridDim.x) {
+#pragma unroll
+          for (int k = 0; k < NV; ++k) ok = ll_recv(slots + (size_t)c * kSlotWords + 2 * k, v[k], tag) && ok;
+        }
+        if (__all_sync(0xffffffffu, ok)) break;
+        const unsigned long long now = global_ns();
+        if (spins++ == 0u) t0 = now;
+        bool stop = (spins & 31u) == 0u && ld_relaxed_i32(&ctl->abort);
+        if ((long long)(now - t0) > timeout_ns) {
+          record_error(ctl, LAP5CG_ERR_SYNC_TIMEOUT);
+          stop = true;
+        }
+        if (__any_sync(0xffffffffu, stop)) {
+          s_go = 0;
+          break;
+        }
+      }
+      __threadfence();
+      if (aborted) s_go = 0;
+#pragma unroll
+      for (int k = 0; k < NV; ++k) v[k] = warp_sum(v[k]);
+      if (lane == 0) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) red[(RED_POLL + pw) * kMaxVals + k] = v[k];
+      }
+    }
+    __syncthreads();
+    if (pw == kPollWarps - 1) {
+      double s[NV], e[NE];
+#pragma unroll
+      for (int k = 0; k < NV; ++k) {
+        s[k] = red[RED_POLL * kMaxVals + k];
+#pragma unroll
+        for (int j = 1; j < kPollWarps; ++j)
+          if (32 * j < (int)gridDim.x) s[k] += red[(RED_POLL + j) * kMaxVals + k];
+      }
+      post(s, e);
+      if (lane == 0) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) red[RED_TOTAL * kMaxVals + k] = s[k];
+#pragma unroll
+        for (int k = 0; k < NE; ++k) red[RED_EXTRA * kMaxVals + k] = e[k];
+      }
+    }
+  } else if (warp == 0) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
-      double s = lane < nwarps ? red[lane * kMaxVals + k] : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      const double s = warp_sum(lane < nwarps ? red[(RED_WARPS + lane) * kMaxVals + k] : 0.0);
       if (lane == 0) ctl->part[par][blockIdx.x][k] = s;
     }
     if (lane == 0) {
@@ -456,22 +553,40 @@ __device__ __forceinline__ bool grid_reduce(Ctl* ctl, unsigned long long& epoch,
     }
     __syncwarp();
     // sum the CTA slots in a fixed order (identical in every CTA)
+    double t[NV], e[NE];
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
       double s = 0.0;
       for (int c = lane; c < (int)gridDim.x; c += 32) s += *((volatile double*)&ctl->part[par][c][k]);
+      t[k] = warp_sum(s);
+    }
+    post(t, e);
+    if (lane == 0) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) red[32 * kMaxVals + k] = s;
+      for (int k = 0; k < NV; ++k) red[RED_TOTAL * kMaxVals + k] = t[k];
+#pragma unroll
+      for (int k = 0; k < NE; ++k) red[RED_EXTRA * kMaxVals + k] = e[k];
     }
   }
   __syncthreads();
   ++epoch;
   const bool go = s_go != 0;
 #pragma unroll
-  for (int k = 0; k < NV; ++k) out[k] = red[32 * kMaxVals + k];
+  for (int k = 0; k < NV; ++k) out[k] = red[RED_TOTAL * kMaxVals + k];
+#pragma unroll
+  for (int k = 0; k < NE; ++k) ex[k] = red[RED_EXTRA * kMaxVals + k];
   __syncthreads();  // red is reused by the next call
   return go;
+}
+
+// The totals alone, from per-thread contributions v[].
+template <int NV>
+__device__ __forceinline__ bool grid_reduce(Ctl* ctl, unsigned long long& epoch, const double (&v)[NV],
+                                            double (&out)[NV], double* red, long long timeout_ns) {
+  double w[NV], ex[1];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) w[k] = warp_sum(v[k]);
+  return grid_reduce_post<NV, 1>(ctl, epoch, w, out, ex, red, timeout_ns, NoScalars());
 }
 
 // Plain grid barrier (no values), same protocol as grid_reduce.
@@ -560,10 +675,8 @@ __host__ __device__ inline Units make_units(int nx, int ny, int V, long long W, 
   return u;
 }
 
-// Shared scratch every solve body needs: per-warp partials (32 x kMaxVals),
-// totals (kMaxVals) and, for cluster teams, the CTA partial by parity
-// (2 x kMaxVals).
-constexpr int kRedDoubles = 35 * kMaxVals;
+// Shared scratch every solve body needs.
+constexpr int kRedDoubles = RED_ROWS * kMaxVals;
 
 // A team is the set of CTAs that solve one system together.
 //  GridTeam: every CTA of a cooperative launch; the barrier is the bounded
@@ -581,6 +694,11 @@ struct GridTeam {
   __device__ __forceinline__ bool reduce(const double (&v)[NV], double (&o)[NV], double* red) {
     return grid_reduce<NV>(ctl, epoch, v, o, red, timeout_ns);
   }
+  template <int NV, int NE, class Post>
+  __device__ __forceinline__ bool reduce_post(const double (&w)[NV], double (&o)[NV], double (&ex)[NE], double* red,
+                                              Post post) {
+    return grid_reduce_post<NV, NE>(ctl, epoch, w, o, ex, red, timeout_ns, post);
+  }
   __device__ __forceinline__ bool sync(double* red) { return grid_sync(ctl, epoch, red, timeout_ns); }
 };
 
@@ -597,23 +715,26 @@ struct ClusterTeam {
   __device__ __forceinline__ void barrier() { cooperative_groups::this_cluster().sync(); }
   template <int NV>
   __device__ __forceinline__ bool reduce(const double (&v)[NV], double (&out)[NV], double* red) {
+    double w[NV], ex[1];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) w[k] = warp_sum(v[k]);
+    return reduce_post<NV, 1>(w, out, ex, red, NoScalars());
+  }
+  template <int NV, int NE, class Post>
+  __device__ __forceinline__ bool reduce_post(const double (&w)[NV], double (&out)[NV], double (&ex)[NE], double* red,
+                                              Post post) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int par = (int)(epoch & 1ull);
-    double* slot = red + 33 * kMaxVals + par * kMaxVals;
+    double* slot = red + (RED_CLUSTER + par) * kMaxVals;
+    if (lane == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double s = v[k];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) red[warp * kMaxVals + k] = s;
+      for (int k = 0; k < NV; ++k) red[(RED_WARPS + warp) * kMaxVals + k] = w[k];
     }
     __syncthreads();
     if (warp == 0) {
 #pragma unroll
       for (int k = 0; k < NV; ++k) {
-        double s = lane < nwarps ? red[lane * kMaxVals + k] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        const double s = warp_sum(lane < nwarps ? red[(RED_WARPS + lane) * kMaxVals + k] : 0.0);
         if (lane == 0) slot[k] = s;
       }
     }
@@ -621,18 +742,22 @@ struct ClusterTeam {
     if (warp == 0) {
       auto cl = cooperative_groups::this_cluster();
       const int n = (int)cl.num_blocks();
+      double t[NV], e[NE];
 #pragma unroll
-      for (int k = 0; k < NV; ++k) {
-        double s = 0.0;
-        if (lane < n) s = *cl.map_shared_rank(slot + k, (unsigned)lane);
+      for (int k = 0; k < NV; ++k) t[k] = warp_sum(lane < n ? *cl.map_shared_rank(slot + k, (unsigned)lane) : 0.0);
+      post(t, e);
+      if (lane == 0) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) red[32 * kMaxVals + k] = s;
+        for (int k = 0; k < NV; ++k) red[RED_TOTAL * kMaxVals + k] = t[k];
+#pragma unroll
+        for (int k = 0; k < NE; ++k) red[RED_EXTRA * kMaxVals + k] = e[k];
       }
     }
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < NV; ++k) out[k] = red[32 * kMaxVals + k];
+    for (int k = 0; k < NV; ++k) out[k] = red[RED_TOTAL * kMaxVals + k];
+#pragma unroll
+    for (int k = 0; k < NE; ++k) ex[k] = red[RED_EXTRA * kMaxVals + k];
     __syncthreads();
     ++epoch;
     return true;

@@ -34,12 +34,14 @@ size_t ws_bytes_ir(int nx, int ny, int variant, int precision) {
 }
 
 template <class TR, int V>
-static int solve_ir_t(const SolvePlan& p, cudaStream_t st) {
+static int solve_ir_t(const SolvePlan& plan, cudaStream_t st) {
+  SolvePlan p = plan;
+  p.opts = with_warps(plan.opts, ring_slot_ir(V, (int)sizeof(TR)));
   const int ldi = inner_ld(p.nx);
   const size_t vr = align_up((size_t)p.ny * ldi * sizeof(TR), kAlign);
   const size_t vf = align_up((size_t)p.ny * ldi * 4, kAlign);
   unsigned char* base = p.ws + kCtlBytes;
-  if (cudaMemsetAsync(p.ws, 0, 256, st) != cudaSuccess) return LAP5CG_ERR_CUDA;
+  if (cudaMemsetAsync(p.ws, 0, kCtlZeroBytes, st) != cudaSuccess) return LAP5CG_ERR_CUDA;
   LaunchCfg cfg;
   RingGeom rg;
   size_t dyn = 0;

@@ -214,7 +214,7 @@ __device__ void ir_solve(const IrArgs<TR>& a, Team& tm, double* red, unsigned ch
         const bool first = (k == 0);
         const Grid<TR> pold = cur ? a.p1 : a.p0;
         const Grid<TR> pnew = cur ? a.p0 : a.p1;
-        double pz;
+        double pz, al[2];
         {  // phase P
           Acc acc;
           const float bm = (float)beta;
@@ -299,13 +299,21 @@ __device__ void ir_solve(const IrArgs<TR>& a, Team& tm, double* red, unsigned ch
             march<V, float, D>(y0, y1, wk.rev(), field, load, finish);
           }
           ++wk.pc;
-          double v[1] = {acc.value()}, o[1];
-          if (!tm.template reduce<1>(v, o, red)) { aborted = true; goto done; }
+          const double w[1] = {warp_sum(acc)}, gm = gamma;
+          double o[1];
+          // alpha, and beside it in lane 1 the reciprocal that the next beta starts from
+          auto post = [gm](const double (&s)[1], double (&e)[2]) {
+            const bool l1 = (threadIdx.x & 31) == 1;
+            const double q = (l1 ? 1.0 : gm) / (l1 ? gm : s[0]);
+            e[0] = __shfl_sync(0xffffffffu, q, 0);
+            e[1] = __shfl_sync(0xffffffffu, q, 1);
+          };
+          if (!tm.template reduce_post<1, 2>(w, o, al, red, post)) { aborted = true; goto done; }
           pz = o[0];
         }
-        if (!(pz > 0.0) || !isfinite(pz)) { status = LAP5CG_ERR_BREAKDOWN; goto done; }
+        if (!bits_positive(pz) || !bits_finite(pz)) { status = LAP5CG_ERR_BREAKDOWN; goto done; }
         {  // phase R
-          const float am = (float)(gamma / pz);
+          const float am = (float)al[0];
           Acc acc, aro;  // (r, r) and, for bf16 storage, (r_new, r_old)
           if (R && !zs) {
             const RingVec vv[3] = {
@@ -397,15 +405,19 @@ __device__ void ir_solve(const IrArgs<TR>& a, Team& tm, double* red, unsigned ch
           }
           ++wk.pc;
           constexpr int NR = kPR ? 2 : 1;
-          double v[NR], o[NR];
-          v[0] = acc.value();
-          if constexpr (kPR) v[NR - 1] = aro.value();
-          if (!tm.template reduce<NR>(v, o, red)) { aborted = true; goto done; }
+          double w[NR], o[NR], be[1];
+          w[0] = warp_sum(acc);
+          if constexpr (kPR) w[NR - 1] = warp_sum(aro);
+          const double gm = gamma, rg = al[1];
+          auto post = [gm, rg](const double (&s)[NR], double (&e)[1]) {
+            e[0] = quotient(kPR ? s[0] - s[NR - 1] : s[0], gm, rg);
+          };
+          if (!tm.template reduce_post<NR, 1>(w, o, be, red, post)) { aborted = true; goto done; }
           const double gnew = o[0];
           ++k;
           ++total;
-          if (!isfinite(gnew)) { status = LAP5CG_ERR_BREAKDOWN; goto done; }
-          beta = (kPR ? gnew - o[NR - 1] : gnew) / gamma;
+          if (!bits_finite(gnew)) { status = LAP5CG_ERR_BREAKDOWN; goto done; }
+          beta = be[0];
           gamma = gnew;
           cur ^= 1;
         }

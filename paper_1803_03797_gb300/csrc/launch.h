@@ -114,6 +114,9 @@ int choose_ring(const void* func, int slot_bytes, const lap5cg_opts& o, int wpc,
 
 // Warps per CTA of the single-grid kernels for these options.
 int warps_of(const lap5cg_opts& o);
+// The options with warps_per_cta filled in for a kernel with ring slots of
+// slot_bytes: the default, or fewer where an explicit ring_slots would not fit.
+lap5cg_opts with_warps(const lap5cg_opts& o, int slot_bytes);
 
 // Largest ring slot (bytes) of each kernel family, V = lane vector width.
 inline int ring_slot_classic(int V, int es) {
@@ -129,7 +132,7 @@ inline int ring_slot_ir(int V, int es_r) {
 }
 
 // Launch defaults (measured on GB300; the autotuner can override them).
-constexpr int kDefaultWarps = 4;          // warps per CTA
+constexpr int kDefaultWarps = 16;         // warps per CTA: one CTA an SM, the reductions' peers
 constexpr int kDefaultMinRows = 2;        // shortest warp unit (rows) on small grids
 constexpr int kRingBytesPerWarp = 12800;  // 16 warps per SM fit 228 KB of shared memory
 constexpr int kRingMinRows = 8;           // automatic ring only for units at least this tall

@@ -530,7 +530,7 @@ template <class TM>
 static int solve_mg_t(const SolvePlan& p, cudaStream_t st) {
   const size_t vec = align_up((size_t)p.ny * (size_t)p.ldw * sizeof(double), kAlign);
   unsigned char* base = p.ws + kCtlBytes;
-  if (cudaMemsetAsync(p.ws, 0, 256, st) != cudaSuccess) return LAP5CG_ERR_CUDA;
+  if (cudaMemsetAsync(p.ws, 0, kCtlZeroBytes, st) != cudaSuccess) return LAP5CG_ERR_CUDA;
   PcgArgs<TM> a;
   int lnx[kMgMaxLevels], lny[kMgMaxLevels];
   a.nlev = mg_levels(p.nx, p.ny, p.opts.mg_levels, lnx, lny);

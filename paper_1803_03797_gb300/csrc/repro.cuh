@@ -294,6 +294,27 @@ __device__ __forceinline__ void acc_discard(Team& tm) {
   }
 }
 
+// Reduce NV accumulators of one kind and form scalars from the totals with
+// post(totals, ex): on one whole warp a CTA, or (exact sums) in every thread.
+template <int NV, int NE, class Team, class Acc, class Post>
+__device__ __forceinline__ bool acc_reduce(Team& tm, Acc* const (&accs)[NV], double (&out)[NV], double (&ex)[NE],
+                                           double* red, Post post) {
+  if constexpr (AccTraits<Acc>::kExact) {
+    if (!grid_reduce_exact<NV>(tm, out, red)) return false;
+    post(out, ex);
+    return true;
+  } else {
+    double w[NV];
+    if constexpr (NV == 2) {
+      warp_sum2(*accs[0], *accs[1], w);
+    } else {
+#pragma unroll
+      for (int k = 0; k < NV; ++k) w[k] = warp_sum(*accs[k]);
+    }
+    return tm.template reduce_post<NV, NE>(w, out, ex, red, post);
+  }
+}
+
 // Reduce NV accumulators of one kind: plain values through the team's
 // reduction, exact ones through grid_reduce_exact.
 template <int NV, class Team, class Acc>
@@ -301,10 +322,8 @@ __device__ __forceinline__ bool acc_reduce(Team& tm, Acc* const (&accs)[NV], dou
   if constexpr (AccTraits<Acc>::kExact) {
     return grid_reduce_exact<NV>(tm, out, red);
   } else {
-    double v[NV];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] = accs[k]->value();
-    return tm.template reduce<NV>(v, out, red);
+    double ex[1];
+    return acc_reduce<NV, 1>(tm, accs, out, ex, red, NoScalars());
   }
 }
 

@@ -27,14 +27,14 @@ static bool res_is_f64(int kind) { return kind == RK_F64_CLASSIC || kind == RK_F
 static bool res_plan(int kind, int nx, int ny, int team, int min_rows, ResPlan* p) {
   const int w = res_is_f64(kind) ? 2 : 4, es = res_is_f64(kind) ? 8 : 4;
   p->groups = ((long long)nx + w - 1) / w;
-  p->rows = res_rows(ny, std::min(team, kResMaxTeam), min_rows);
+  p->rows = res_rows(ny, std::min(team, kMaxPeers), min_rows);
   const long long items = p->groups * p->rows;
   if (items > (long long)res_most_items(kind) * kResMaxThreads) return false;
   p->items = (int)items;
   p->ctas = (ny + p->rows - 1) / p->rows;
   p->k = (int)((items + kResMaxThreads - 1) / kResMaxThreads);
   p->smem = (size_t)(p->rows + 4) * p->groups * w * es;  // two halo rows, two more staged
-  p->slot_bytes = (size_t)2 * p->ctas * kResSlotWords * 8;
+  p->slot_bytes = (size_t)2 * p->ctas * kSlotWords * 8;
   p->halo_bytes = (size_t)4 * p->ctas * p->groups * kResItemWords * 8;
   return true;
 }
@@ -183,7 +183,7 @@ int resident_batched(int count, const int* nx, const int* ny, const int* ld, con
   DevProps dp;
   int rc = dev_props(&dp);
   if (rc != LAP5CG_OK) return rc;
-  const int sms = std::min(dp.sms, kResMaxTeam);
+  const int sms = std::min(dp.sms, kMaxPeers);
   const int min_rows = 3;  // the message memory then fits in the place of the state vectors
   const size_t smem_cap = (size_t)dp.max_smem_optin - sizeof(ResShared) - 1024;
   std::vector<ResPick> picks;
@@ -225,7 +225,7 @@ int resident_batched(int count, const int* nx, const int* ny, const int* ld, con
   const auto c = classes(best);
   // message memory: the abort flag, per launch a queue head and a word a team, then
   // the instances'; all of it starts at zero
-  constexpr size_t kLaunchBytes = 256 + 32 * kResSlotWords * 8;
+  constexpr size_t kLaunchBytes = 256 + 32 * kSlotWords * 8;
   size_t off = first_off + kAlign;
   std::vector<size_t> launch_off(c.size(), 0);
   for (size_t s = 0; s < c.size(); ++s)

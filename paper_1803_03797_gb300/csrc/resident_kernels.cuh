@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) k_resident_batch(const ResB
   __shared__ int s_item;
   extern __shared__ __align__(16) unsigned char dsm[];
   const int team = (int)blockIdx.x / l.team, rank = (int)blockIdx.x - team * l.team;
-  u64* word = l.item + (size_t)team * kResSlotWords;
+  u64* word = l.item + (size_t)team * kSlotWords;
   uint32_t seq = 0;
   for (;;) {
     // The team's first CTA draws an item and passes it on.  A CTA that an
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) k_resident_batch(const ResB
       const int groups = (e.nx + W - 1) / W;
       u64* mem = reinterpret_cast<u64*>(l.ws + e.ws_off);
       ResTeam tm;
-      tm.init(mem, mem + (size_t)2 * ctas * kResSlotWords, rank, ctas, groups, l.errs + e.idx, l.abort_flag,
+      tm.init(mem, mem + (size_t)2 * ctas * kSlotWords, rank, ctas, groups, l.errs + e.idx, l.abort_flag,
               2000000000LL, &sh);
       res_body_of<KIND>((rows * groups + kResMaxThreads - 1) / kResMaxThreads, a, tm, reinterpret_cast<T*>(dsm));
     }
