@@ -150,4 +150,103 @@ __device__ __forceinline__ void march_ring_fix(WarpRing& ring, int ny, int lane,
   ring.q = q0 + (unsigned)total;
 }
 
+// The same march over rows loaded straight into registers: load(j, Raw&) reads row j
+// one step ahead of its use, field(j, raw, FRow&) builds the operand's row from it,
+// finish(j, c, y) consumes row j.
+template <int V, class Raw, class LoadF, class FieldF, class FinishF>
+__device__ __forceinline__ void march_fix(int ny, int lane, int y0, int y1, bool rev, LoadF& load, FieldF& field,
+                                          FinishF& finish) {
+  if (y0 >= y1) return;
+  const int step = rev ? -1 : 1;
+  const int T = y1 - y0, first = rev ? y1 : y0 - 1;
+  FixRow<V> prev, sum;
+  double c[V];
+  Raw next;
+  load(first, next);
+  for (int t = 0; t < T + 2; ++t) {
+    const int j = first + t * step;
+    const Raw cur = next;
+    if (t < T + 1) load(j + step, next);
+    FRow<V, double> f;
+    if (j < 0 || j >= ny) f.zero();
+    else field(j, cur, f);
+    FixRow<V> a;
+    unsigned m = (unsigned)__double2hiint(f.hl) & 0x7fffffffu;
+#pragma unroll
+    for (int k = 0; k < V; ++k) m = max(m, (unsigned)__double2hiint(f.f[k]) & 0x7fffffffu);
+    a.E = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
+#pragma unroll
+    for (int k = 0; k < V; ++k) a.q[k] = fix_of(f.f[k], a.E);
+    if (t >= 2) {
+      const int E = max(sum.E, a.E);
+      fix_align<V>(sum.q, sum.E, E);
+      long long n[V];
+#pragma unroll
+      for (int k = 0; k < V; ++k) n[k] = a.q[k];
+      fix_align<V>(n, a.E, E);
+      double y[V];
+#pragma unroll
+      for (int k = 0; k < V; ++k) y[k] = fix_to(sum.q[k] - n[k], E);
+      if (E < kFixLow || E > kFixHigh) {
+#pragma unroll
+        for (int k = 0; k < V; ++k) y[k] = E < kFixLow ? 0.0 : __longlong_as_double(0x7ff8000000000000ll);
+      }
+      finish(j - step, c, y);
+    }
+    const long long h = fix_of(f.hl, a.E);
+    long long l = __shfl_up_sync(0xffffffffu, a.q[V - 1], 1), r = __shfl_down_sync(0xffffffffu, a.q[0], 1);
+    if (lane == 0) l = h;
+    if (lane == 31) r = h;
+    const int E = t == 0 ? a.E : max(prev.E, a.E);
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      const long long w = k == 0 ? l : a.q[k - 1], e = k == V - 1 ? r : a.q[k + 1];
+      sum.q[k] = 4 * a.q[k] - w - e;
+      c[k] = f.f[k];
+    }
+    if (t > 0) {
+      fix_align<V>(sum.q, a.E, E);
+      fix_align<V>(prev.q, prev.E, E);
+#pragma unroll
+      for (int k = 0; k < V; ++k) sum.q[k] -= prev.q[k];
+    }
+    sum.E = E;
+    prev = a;
+  }
+}
+
+__device__ __forceinline__ unsigned fix_mag(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+
+// r of fixed-point sums q at exponent E (uniform in the warp), the range's ends included.
+template <int V>
+__device__ __forceinline__ void fix_results(const long long (&q)[V], int E, double (&r)[V]) {
+#pragma unroll
+  for (int k = 0; k < V; ++k) r[k] = fix_to(q[k], E);
+  if (E < kFixLow || E > kFixHigh) {
+#pragma unroll
+    for (int k = 0; k < V; ++k) r[k] = E < kFixLow ? 0.0 : __longlong_as_double(0x7ff8000000000000ll);
+  }
+}
+
+// r = b - A c on a lane vector from its neighbours (up, dn: rows; w, e: columns), all
+// aligned to the warp's largest exponent: nine values of that size at most stay
+// below 2^63.  Every lane of the warp calls.
+template <int W>
+__device__ __forceinline__ void fix_residual(const double (&c)[W], const double (&up)[W], const double (&dn)[W],
+                                             double w, double e, const double (&b)[W], double (&r)[W]) {
+  unsigned m = max(fix_mag(w), fix_mag(e));
+#pragma unroll
+  for (int k = 0; k < W; ++k) m = max(max(m, max(fix_mag(c[k]), fix_mag(b[k]))), max(fix_mag(up[k]), fix_mag(dn[k])));
+  const int E = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
+  long long q[W], f[W];
+#pragma unroll
+  for (int k = 0; k < W; ++k) f[k] = fix_of(c[k], E);
+  const long long l = fix_of(w, E), h = fix_of(e, E);
+#pragma unroll
+  for (int k = 0; k < W; ++k)
+    q[k] = fix_of(b[k], E) - 4 * f[k] + (k == 0 ? l : f[k - 1]) + (k == W - 1 ? h : f[k + 1]) + fix_of(up[k], E) +
+           fix_of(dn[k], E);
+  fix_results<W>(q, E, r);
+}
+
 }  // namespace lap5

@@ -16,15 +16,20 @@
 //
 // The host replays the V-cycle's pass sequence (Vcycle::run in mg_kernels.cuh:
 // which buffer each pass reads and writes, the march direction) into one
-// kernel node per pass; the levels of at most kMgCtaPoints points run in one
+// kernel node per pass; for nu = 2 the levels that fit in the SMs' shared memory
+// (from 1023^2 down at 4096^2, binary32) run in one cooperative kernel node
+// (mg_mid.cuh), otherwise those of at most kMgCtaPoints points in one
 // single-CTA kernel node.  Instantiated graphs are cached per call signature
 // (device, shape, workspace, V-cycle options; lap5cg_release_graphs frees
 // them all); a small kernel writes each call's b, x, info, history, tol and
 // maxit into the workspace before the cached graph is launched.
+#include <algorithm>
 #include <mutex>
 #include <vector>
 
+#include "fixstencil.cuh"
 #include "mg_kernels.cuh"
+#include "mg_mid.cuh"
 
 namespace lap5 {
 
@@ -33,7 +38,7 @@ constexpr int kGmMaxBlocks = 4096;  // partial-sum slots
 
 // Solve state in device memory (the workspace's control block).
 struct GmScal {
-  double bb, thr, rr, gamma, alpha, beta;
+  double bb, thr, rr, gamma[2], alpha;  // gamma: by iteration parity
   int iters, status, stop, cur, zero_x;
   int xpend;  // x += alpha p of the last x, r pass is still to be applied (k_gm_pq or k_gm_xfinal)
 };
@@ -57,27 +62,21 @@ __global__ void k_gm_bind(GmBind* bd, const double* b, double* x, lap5cg_info* i
 
 enum { GP_JAC = 0, GP_JAC_DOT, GP_RES, GP_RESTRICT, GP_PROLONG, GP_RES_RESTRICT, GP_PROLONG_JAC, GP_JAC_RES_RESTRICT };
 
-// Block-wide sums of NV per-thread values into part[blockIdx.x * 2 + k].
+// Block-wide sums of NV per-thread values into part[blockIdx.x * 2 + k] (sums over
+// lanes in fixed point: exchange.cuh).
 template <int NV>
 __device__ __forceinline__ void gm_partials(const double (&v)[NV], double* part) {
   __shared__ double sred[32][2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
-    double s = v[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const double s = warp_sum(v[k]);
     if (lane == 0) sred[warp][k] = s;
   }
   __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double s = lane < nw ? sred[lane][k] : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) part[blockIdx.x * 2 + k] = s;
-    }
+  if (warp < NV) {
+    const double s = warp_sum(lane < nw ? sred[lane][warp] : 0.0);
+    if (lane == 0) part[blockIdx.x * 2 + warp] = s;
   }
 }
 
@@ -89,14 +88,11 @@ __device__ __forceinline__ double gm_total(const double* part, int nb, int k) {
   double s = 0.0;
   for (int b = threadIdx.x; b < nb; b += blockDim.x) s += part[b * 2 + k];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  s = warp_sum(s);
   if (lane == 0) sw[warp] = s;
   __syncthreads();
   if (warp == 0) {
-    double t = lane < nw ? sw[lane] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    const double t = warp_sum(lane < nw ? sw[lane] : 0.0);
     if (lane == 0) total = t;
   }
   __syncthreads();
@@ -178,15 +174,57 @@ __global__ void __launch_bounds__(kGmThreads) k_gm_sweep(const GmScal* sc, doubl
         for (int q = 0; q < V; ++q) bv[k][q] = TM(0);
       }
     }
+    TM rs[R][V];  // b - A u
+    if constexpr (sizeof(TM) == 8) {
+      // binary64: in fixed point over the tile's rows (fixstencil.cuh), one FP64
+      // operation a point instead of five
+      unsigned m = 0u;
+#pragma unroll
+      for (int k = 0; k < R + 2; ++k) {
+#pragma unroll
+        for (int q = 0; q < V; ++q) m = max(m, fix_mag(f[k].f[q]));
+        if (k >= 1 && k <= R) {
+          m = max(m, max(fix_mag(f[k].hl), fix_mag(f[k].hr)));
+#pragma unroll
+          for (int q = 0; q < V; ++q) m = max(m, fix_mag(bv[k - 1][q]));
+        }
+      }
+      const int E = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
+      long long w[R + 2][V];
+#pragma unroll
+      for (int k = 0; k < R + 2; ++k)
+#pragma unroll
+        for (int q = 0; q < V; ++q) w[k][q] = fix_of(f[k].f[q], E);
+#pragma unroll
+      for (int k = 0; k < R; ++k) {
+        const long long h = fix_of(lane == 0 ? f[k + 1].hl : f[k + 1].hr, E);
+        long long l = __shfl_up_sync(0xffffffffu, w[k + 1][V - 1], 1);
+        long long r = __shfl_down_sync(0xffffffffu, w[k + 1][0], 1);
+        if (lane == 0) l = h;
+        if (lane == 31) r = h;
+        long long d[V];
+#pragma unroll
+        for (int q = 0; q < V; ++q)
+          d[q] = fix_of(bv[k][q], E) - 4 * w[k + 1][q] + (q == 0 ? l : w[k + 1][q - 1]) +
+                 (q == V - 1 ? r : w[k + 1][q + 1]) + w[k][q] + w[k + 2][q];
+        fix_results<V>(d, E, rs[k]);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < R; ++k) {
+        TM ax[V];
+        stencil_row<V>(f[k], f[k + 1], f[k + 2], lane, ax);
+#pragma unroll
+        for (int q = 0; q < V; ++q) rs[k][q] = bv[k][q] - ax[q];
+      }
+    }
 #pragma unroll
     for (int k = 0; k < R; ++k) {
       const int j = jb + k;
       if (j >= L.ny) break;
-      TM ax[V], o[V];
-      stencil_row<V>(f[k], f[k + 1], f[k + 2], lane, ax);
+      TM o[V];
 #pragma unroll
-      for (int q = 0; q < V; ++q)
-        o[q] = MODE == GP_RES ? bv[k][q] - ax[q] : mg_fma(c, bv[k][q] - ax[q], f[k + 1].f[q]);
+      for (int q = 0; q < V; ++q) o[q] = MODE == GP_RES ? rs[k][q] : mg_fma(c, rs[k][q], f[k + 1].f[q]);
       store_row<V>(go, j, xl, L.nx, o);
       if constexpr (MODE == GP_JAC_DOT) {
         double rv[V], zv[V];
@@ -622,6 +660,97 @@ __global__ void __launch_bounds__(512) k_gm_small(const GmScal* sc, GmLevels<TM>
   gm_small_levels<TM, SMEM>(levels, nlev, first, nu, nu_c, gsm, lv);
 }
 
+// The levels from m.lv[0] on (mg_mid.cuh): m.n distributed ones, then
+// [small_first, nlev) on the last CTA.
+template <class TM>
+__global__ void __launch_bounds__(kMidThreads, 1) k_gm_mid(GmScal* sc, MidArgs<TM> m, GmLevels<TM> levels, int nlev,
+                                                           int small_first, int nu_c) {
+  if (sc->stop) return;
+  extern __shared__ __align__(16) unsigned char gsm[];
+  TM* sm = reinterpret_cast<TM*>(gsm);
+  const int cta = (int)blockIdx.x, tag = sc->iters + 1, n = m.n;
+  auto flags = [&](int stage) { return m.flags + stage * kMidMaxCtas; };
+  auto fail = [&]() {
+    if (threadIdx.x == 0) {
+      sc->status = LAP5CG_ERR_SYNC_TIMEOUT;
+      sc->stop = 1;
+    }
+  };
+  // stages: [1, n] b of distributed level 1 .. n - 1 and of the small levels
+  // written; n + 1 the small levels' result; n + 1 + l the result of level n - l
+  if (cta == (int)gridDim.x - 1) {
+    for (int i = threadIdx.x; i < tiny_elems<TM>(levels.lv, small_first, nlev); i += blockDim.x) sm[i] = TM(0);
+    if (!mid_wait(flags(n), 0, m.lv[n - 1].G - 1, tag, m.abort_flag)) return fail();
+    tiny_levels<TM>(levels.lv, small_first, nlev, nu_c, sm, levels.lv[small_first].u);
+    mid_signal(flags(n + 1), tag);
+    return;
+  }
+  for (size_t i = threadIdx.x; i < (size_t)m.offE; i += blockDim.x) sm[i] = TM(0);  // pads stay zero
+  __syncthreads();
+  auto below = [&](int l) -> const MgLevel<TM>& { return l + 1 < n ? m.lv[l + 1].g : levels.lv[small_first]; };
+  for (int l = 0; l < n; ++l) {
+    const MidLevel<TM>& L = m.lv[l];
+    if (cta >= L.G) continue;
+    const int s = cta * L.R, e = min(L.g.ny, s + L.R);
+    if (l > 0) {  // the owners of the centre rows of b rows s - 3 .. e + 2
+      const MidLevel<TM>& F = m.lv[l - 1];
+      const int j0 = 2 * max(s - 3, 0) + 1, j1 = 2 * min(e + 2, L.g.ny - 1) + 1;
+      if (!mid_wait(flags(l), j0 / F.R, j1 / F.R, tag, m.abort_flag)) return fail();
+    }
+    mid_down<TM>(L, below(l), sm, m.offT, cta);
+    mid_signal(flags(l + 1) + cta, tag);
+  }
+  for (int l = n - 1; l >= 0; --l) {
+    const MidLevel<TM>& L = m.lv[l];
+    if (cta >= L.G) continue;
+    const int s = cta * L.R, e = min(L.g.ny, s + L.R);
+    const TM* eg;
+    TM* E;
+    if (l == n - 1) {
+      if (!mid_wait(flags(n + 1), 0, 0, tag, m.abort_flag)) return fail();
+      eg = levels.lv[small_first].u;
+      E = sm + m.offE;
+    } else {
+      const MidLevel<TM>& C = m.lv[l + 1];
+      const int J0 = max(((s - 2) >> 1) - 1, 0), J1 = min((e + 1) >> 1, C.g.ny - 1);
+      if (!mid_wait(flags(2 * n - l), J0 / C.R, J1 / C.R, tag, m.abort_flag)) return fail();
+      eg = C.g.u;
+      E = sm + C.offB;  // that level is done: its rows take the correction
+    }
+    mid_up<TM>(L, below(l), eg, E, sm, m.offT, L.g.u, cta);
+    if (l > 0) mid_signal(flags(2 * n + 1 - l) + cta, tag);
+  }
+}
+
+// Splits the levels from `first` on over at most ctas - 1 CTAs; false when they do
+// not fit.  Fills m (but for the pointers to the control block) and the
+// first level of the last CTA.
+template <class TM>
+static bool gm_mid_plan(const PcgArgs<TM>& a, int first, int ctas, size_t smem_cap, MidArgs<TM>* m, int* small_first,
+                        int* grid, size_t* smem) {
+  if (a.nu != 2 || first < 1) return false;
+  int ls = first;
+  while (ls < a.nlev && (long long)a.lv[ls].nx * a.lv[ls].ny > kMidSmallPoints<TM>) ++ls;
+  if (ls >= a.nlev || ls == first || ls - first > kMidMaxLevels) return false;
+  const int most = std::min(ctas, kMidMaxCtas) - 1;
+  m->n = ls - first;
+  *grid = 0;
+  for (int l = first; l < ls; ++l) {
+    MidLevel<TM>& L = m->lv[l - first];
+    L.g = a.lv[l];
+    L.R = (L.g.ny + most - 1) / most;
+    L.G = (L.g.ny + L.R - 1) / L.R;
+    *grid = std::max(*grid, L.G);
+  }
+  ++*grid;
+  *small_first = ls;
+  *smem = std::max(mid_layout<TM>(m, a.lv[ls]), tiny_elems<TM>(a.lv, ls, a.nlev) * sizeof(TM));
+  // a level's rows take the next coarser correction: R/2 + 4 rows of it at most
+  for (int k = 0; k + 1 < m->n; ++k)
+    if ((m->lv[k].R + 4) / 2 + 4 > m->lv[k + 1].R + 6 + m->lv[k + 1].R + 4) return false;
+  return *smem + 4096 <= smem_cap;
+}
+
 // r = b - A x, level 0: b = r (rounded to TM), u = c b (write_u); partials
 // (b, b), (r, r).
 template <class TM>
@@ -664,7 +793,7 @@ __global__ void __launch_bounds__(kGmThreads) k_gm_init(const GmBind* bd, double
 #pragma unroll
       for (int k = 0; k < V; ++k) {
         rv[k] = d.b[k] - ax[k];
-        rb[k] = (TM)rv[k];
+        rb[k] = mg_narrow<TM>(rv[k]);
         ru[k] = cm * rb[k];
       }
       acc_dot<V>(abb, j, d.b, d.b, nval);
@@ -681,7 +810,8 @@ __global__ void __launch_bounds__(kGmThreads) k_gm_init(const GmBind* bd, double
 
 // (b, b), (r, r) -> threshold, status; the loop's condition.
 __global__ void __launch_bounds__(256) k_gm_start(GmScal* sc, const GmBind* bd, const double* part, int nb,
-                                                  cudaGraphConditionalHandle h) {
+                                                  cudaGraphConditionalHandle h, int* flags) {
+  for (int i = threadIdx.x; i < kMidStages * kMidMaxCtas + 1; i += blockDim.x) flags[i] = 0;  // k_gm_mid's
   const double tol = bd->tol;
   const int maxit = bd->maxit;
   double* history = bd->history;
@@ -709,33 +839,40 @@ __global__ void __launch_bounds__(256) k_gm_start(GmScal* sc, const GmBind* bd, 
   cudaGraphSetConditional(h, s.stop ? 0u : 1u);
 }
 
-// (r, z) -> beta, gamma (breakdown if not positive).
-__global__ void __launch_bounds__(256) k_gm_rz(GmScal* sc, const double* part, int nb) {
-  if (sc->stop) return;
-  const double rz = gm_total(part, nb, 0);
-  if (threadIdx.x != 0) return;
-  if (!(rz > 0.0) || !isfinite(rz)) {
-    sc->status = LAP5CG_ERR_BREAKDOWN;
-    sc->stop = 1;
-    return;
-  }
-  sc->beta = (sc->iters == 0) ? 0.0 : rz / sc->gamma;
-  sc->gamma = rz;
-}
-
 // p = z + beta p (halo included), q = A p, partial (p, q); and the previous
 // iteration's x += alpha p with that p (read here anyway), deferred from the
-// x, r pass (which then moves 16 bytes a point fewer).
+// x, r pass (which then moves 16 bytes a point fewer).  Every CTA forms beta from the
+// (r, z) sweep's nbz partial sums: a kernel of its own for it cost 4 us an iteration,
+// the sums (one load a thread, fixed point) 0.6 us.  gamma alternates between two
+// places, since CTA 0 stores the new one while others may still read the old.
 template <class TM>
-__global__ void __launch_bounds__(kGmThreads) k_gm_pq(const GmScal* sc, const GmBind* bd, double* part, int nx,
-                                                       int ny, int ld, Grid<double> p0, Grid<double> p1,
-                                                       Grid<double> q, MgLevel<TM> L0, int zbuf, int rev) {
+__global__ void __launch_bounds__(kGmThreads) k_gm_pq(GmScal* sc, const GmBind* bd, const double* partz, int nbz,
+                                                       double* part, int nx, int ny, int ld, Grid<double> p0,
+                                                       Grid<double> p1, Grid<double> q, MgLevel<TM> L0, int zbuf,
+                                                       int rev) {
   if (sc->stop) return;
   constexpr int V = 2;
   const Sched s = gm_sched(rev);
   const Units un = make_units(nx, ny, V, s.nw, 2);
-  const double beta = sc->beta;
-  const bool first = (sc->iters == 0);
+  const int iters = sc->iters;
+  const bool first = (iters == 0);
+  __shared__ double s_beta;
+  {
+    const double rz = gm_total(partz, nbz, 0);
+    if (!bits_positive(rz) || !bits_finite(rz)) {  // (the same in every CTA)
+      if (blockIdx.x == 0 && threadIdx.x == 0) {
+        sc->status = LAP5CG_ERR_BREAKDOWN;
+        sc->stop = 1;
+      }
+      return;
+    }
+    if (threadIdx.x == 0) {
+      s_beta = first ? 0.0 : rz / sc->gamma[(iters & 1) ^ 1];
+      if (blockIdx.x == 0) sc->gamma[iters & 1] = rz;
+    }
+    __syncthreads();
+  }
+  const double beta = s_beta;
   const bool xp = sc->xpend != 0;
   const double alpha_old = sc->alpha;
   const Grid<double> x{bd->x, ld};
@@ -743,84 +880,88 @@ __global__ void __launch_bounds__(kGmThreads) k_gm_pq(const GmScal* sc, const Gm
   const Grid<double> pnew = sc->cur ? p0 : p1;
   const Grid<const TM> gz{zbuf ? L0.v : L0.u, L0.ld};
   Acc64 apq;
-  struct D { double x[V], p[V]; };
+  struct Raw {
+    TM z[V], zh;
+    double p[V], ph, x[V];
+  };
   for (int u = s.w; u < un.nunits; u += s.nw) {
     int st, y0, y1;
     unit_bounds(un, u, ny, st, y0, y1);
     const int xs = st * 32 * V, xl = Lanes<V>::first(xs, s.lane);
     const int nval = nx - xl;
-    auto zone = [&](int j, int xx) -> double { return (xx < 0 || xx >= nx) ? 0.0 : mg_widen(gz.row(j)[xx]); };
-    auto pone = [&](int j, int xx) -> double { return (xx < 0 || xx >= nx) ? 0.0 : pold.row(j)[xx]; };
-    auto field = [&](int j, FRow<V, double>& f) {
-      if (j < 0 || j >= ny) { f.zero(); return; }
-      TM zt[V];
-      load_row<V>(gz, j, xl, nx, zt);
-      if (first) {
+    const int xh = s.lane == 0 ? xs - 1 : xs + 32 * V;  // the halo column of lanes 0 and 31
+    const bool halo = (s.lane == 0 || s.lane == 31) && xh >= 0 && xh < nx;
+    auto load = [&](int j, Raw& w) {
+      w.zh = TM(0);
+      w.ph = 0.0;
 #pragma unroll
-        for (int k = 0; k < V; ++k) f.f[k] = mg_widen(zt[k]);
-        f.hl = (s.lane == 0) ? zone(j, xs - 1) : 0.0;
-        f.hr = (s.lane == 31) ? zone(j, xs + 32 * V) : 0.0;
-      } else {
-        double pv[V];
-        load_row<V>(pold, j, xl, nx, pv);
+      for (int k = 0; k < V; ++k) w.p[k] = 0.0;
+      if (j < 0 || j >= ny) return;
+      load_row<V>(gz, j, xl, nx, w.z);
+      if (halo) w.zh = gz.row(j)[xh];
+      if (!first) {
+        load_row<V>(pold, j, xl, nx, w.p);
+        if (halo) w.ph = pold.row(j)[xh];
+      }
+      if (xp && j >= y0 && j < y1) load_row<V>(x, j, xl, nx, w.x);
+    };
+    auto field = [&](int j, const Raw& w, FRow<V, double>& f) {
 #pragma unroll
-        for (int k = 0; k < V; ++k) f.f[k] = __fma_rn(beta, pv[k], mg_widen(zt[k]));
-        f.hl = (s.lane == 0) ? __fma_rn(beta, pone(j, xs - 1), zone(j, xs - 1)) : 0.0;
-        f.hr = (s.lane == 31) ? __fma_rn(beta, pone(j, xs + 32 * V), zone(j, xs + 32 * V)) : 0.0;
-      }
-    };
-    auto load = [&](int j, D& d) {
-      if (xp) {
-        load_row<V>(x, j, xl, nx, d.x);
-        load_row<V>(pold, j, xl, nx, d.p);
-      }
-    };
-    auto finish = [&](int j, const D& d, const FRow<V, double>& S, const FRow<V, double>& C,
-                      const FRow<V, double>& N) {
-      double qv[V];
-      stencil_row<V>(S, C, N, s.lane, qv);
-      store_row<V>(pnew, j, xl, nx, C.f);
-      store_row<V>(q, j, xl, nx, qv);
-      acc_dot<V>(apq, j, C.f, qv, nval);
-      if (xp) {
+      for (int k = 0; k < V; ++k) f.f[k] = __fma_rn(beta, w.p[k], mg_widen(w.z[k]));
+      f.hl = f.hr = __fma_rn(beta, w.ph, mg_widen(w.zh));
+      if (xp && j >= y0 && j < y1) {
         double xv[V];
 #pragma unroll
-        for (int k = 0; k < V; ++k) xv[k] = __fma_rn(alpha_old, d.p[k], d.x[k]);
+        for (int k = 0; k < V; ++k) xv[k] = __fma_rn(alpha_old, w.p[k], w.x[k]);
         store_row<V>(x, j, xl, nx, xv);
       }
     };
-    march<V, double, D>(y0, y1, s.rev, field, load, finish);
+    auto finish = [&](int j, const double (&pv)[V], const double (&qv)[V]) {
+      store_row<V>(pnew, j, xl, nx, pv);
+      store_row<V>(q, j, xl, nx, qv);
+      acc_dot<V>(apq, j, pv, qv, nval);
+    };
+    march_fix<V, Raw>(ny, s.lane, y0, y1, s.rev, load, field, finish);
   }
   const double v[1] = {apq.value()};
   gm_partials<1>(v, part);
 }
 
-// (p, q) -> alpha (breakdown if not positive); the new p becomes current.
-__global__ void __launch_bounds__(256) k_gm_alpha(GmScal* sc, const double* part, int nb) {
-  if (sc->stop) return;
-  const double pq = gm_total(part, nb, 0);
-  if (threadIdx.x != 0) return;
-  sc->xpend = 0;  // k_gm_pq applied the previous x update
-  if (!(pq > 0.0) || !isfinite(pq)) {
-    sc->status = LAP5CG_ERR_BREAKDOWN;
-    sc->stop = 1;
-    return;
-  }
-  sc->alpha = sc->gamma / pq;
-  sc->cur ^= 1;
-}
-
 // r -= alpha q, partial (r, r); level 0: b = r, u = c b (write_u).  (x += alpha p
-// is left to the next p, q pass or, after the loop, to k_gm_xfinal.)
+// is left to the next p, q pass or, after the loop, to k_gm_xfinal.)  Every CTA
+// forms alpha from the p, q pass's nbq partial sums; CTA 0 records it, and that the
+// new p is current and the previous x update done.
 template <class TM>
-__global__ void __launch_bounds__(kGmThreads) k_gm_xr(const GmScal* sc, double* part, int nx, int ny,
+__global__ void __launch_bounds__(kGmThreads) k_gm_xr(GmScal* sc, const double* partq, int nbq, double* part, int nx,
+                                                       int ny,
                                                        Grid<double> r, Grid<double> q, MgLevel<TM> L0, int rev,
                                                        int write_u) {
   if (sc->stop) return;
   constexpr int V = 2;
   const Sched s = gm_sched(rev);
   const Units un = make_units(nx, ny, V, s.nw, 2);
-  const double alpha = sc->alpha;
+  __shared__ double s_alpha;
+  {
+    const double pq = gm_total(partq, nbq, 0);
+    const bool ok = bits_positive(pq) && bits_finite(pq);  // (the same in every CTA)
+    if (threadIdx.x == 0) {
+      const double al = ok ? sc->gamma[sc->iters & 1] / pq : 0.0;
+      s_alpha = al;
+      if (blockIdx.x == 0) {
+        sc->xpend = 0;
+        if (ok) {
+          sc->alpha = al;
+          sc->cur ^= 1;
+        } else {
+          sc->status = LAP5CG_ERR_BREAKDOWN;
+          sc->stop = 1;
+        }
+      }
+    }
+    if (!ok) return;
+    __syncthreads();
+  }
+  const double alpha = s_alpha;
   const Grid<TM> g0b{L0.b, L0.ld}, g0u{L0.u, L0.ld};
   const TM cm = (TM)kMgC;
   Acc64 arr;
@@ -840,7 +981,7 @@ __global__ void __launch_bounds__(kGmThreads) k_gm_xr(const GmScal* sc, double* 
 #pragma unroll
       for (int k = 0; k < V; ++k) {
         rv[k] = __fma_rn(-alpha, d.q[k], d.r[k]);
-        rb[k] = (TM)rv[k];
+        rb[k] = mg_narrow<TM>(rv[k]);
         ru[k] = cm * rb[k];
       }
       acc_dot<V>(arr, j, rv, rv, nval);
@@ -973,10 +1114,11 @@ struct GmPassRec {
 // level's first reader of its first sweep c b is a Jacobi sweep (*write_u =
 // false), that sweep forms c b from b and no producer stores it.  (A binary64
 // V-cycle keeps the separate passes: its fused forms measured slower, the
-// arithmetic, not the traffic, being its limit.)  Returns the buffer that
-// holds level 0's result (M^-1 r).
+// arithmetic, not the traffic, being its limit.)  mid > 0: the levels from it on
+// are one entry (kind -2, k_gm_mid).  Returns the buffer that holds level 0's
+// result (M^-1 r).
 template <class TM>
-static int gm_pass_list(const PcgArgs<TM>& a, bool fuse, std::vector<GmPassRec<TM>>& out, bool* write_u) {
+static int gm_pass_list(const PcgArgs<TM>& a, bool fuse, int mid, std::vector<GmPassRec<TM>>& out, bool* write_u) {
   const int L = a.nlev, nu = a.nu;
   *write_u = !fuse || nu < 2 || (a.lsmall >= L && a.nu_c < 2);
   const int fb = *write_u ? 0 : 1;
@@ -991,7 +1133,7 @@ static int gm_pass_list(const PcgArgs<TM>& a, bool fuse, std::vector<GmPassRec<T
   auto sweeps = [&](int l, int n, bool final0) {  // sweeps 2 .. n (the first, c b, came with b)
     for (int k = 1; k < n; ++k) jac(l, final0 && l == 0 && k == n - 1, k == 1 ? fb : 0);
   };
-  const int big_end = a.lsmall < L - 1 ? a.lsmall : L - 1;
+  const int big_end = mid > 0 ? mid : a.lsmall < L - 1 ? a.lsmall : L - 1;
   for (int l = 0; l < big_end; ++l) {  // down: pre-smoothing, residual, restriction
     if (fuse && nu == 2) {  // the one explicit sweep, residual and restriction: one pass
       out.push_back({GP_JAC_RES_RESTRICT, l, (int)(pc++ & 1u), nullptr, other(l), nullptr});
@@ -1008,7 +1150,10 @@ static int gm_pass_list(const PcgArgs<TM>& a, bool fuse, std::vector<GmPassRec<T
     }
     cur[l + 1] = 0;
   }
-  if (a.lsmall >= L) {
+  if (mid > 0) {
+    out.push_back({-2, big_end, 0, nullptr, nullptr, nullptr});
+    cur[big_end] = 0;
+  } else if (a.lsmall >= L) {
     sweeps(L - 1, a.nu_c, false);
   } else {
     out.push_back({-1, big_end, 0, nullptr, nullptr, nullptr});
@@ -1066,7 +1211,7 @@ static int gm_blocks(const void* fn, int threads, int sms) {
 }
 
 template <class TM>
-static int gm_build(const SolvePlan& p, const PcgArgs<TM>& a, cudaGraphExec_t* exec) {
+static int gm_build(const SolvePlan& p, const PcgArgs<TM>& a, bool use_mid, cudaGraphExec_t* exec) {
   DevProps dp;
   int rc = dev_props(&dp);
   if (rc != LAP5CG_OK) return rc;
@@ -1100,7 +1245,17 @@ static int gm_build(const SolvePlan& p, const PcgArgs<TM>& a, cudaGraphExec_t* e
   const int nb_true = gm_blocks(f_true, kGmThreads, dp.sms);
   std::vector<GmPassRec<TM>> passes;
   bool wu = true;
-  const int zbuf = gm_pass_list<TM>(a, sizeof(TM) == 4, passes, &wu);
+  int* flags = reinterpret_cast<int*>(p.ws + kMidFlagOffset);
+  // the first level from which the rest fits in shared memory
+  MidArgs<TM> mid = {};
+  int mid_first = 0, mid_small = 0, mid_grid = 0;
+  size_t mid_smem = 0;
+  if (use_mid) {
+    for (int l = 1; l < a.nlev && mid_first == 0; ++l)
+      if (gm_mid_plan<TM>(a, l, dp.sms, (size_t)dp.max_smem_optin, &mid, &mid_small, &mid_grid, &mid_smem))
+        mid_first = l;
+  }
+  const int zbuf = gm_pass_list<TM>(a, sizeof(TM) == 4, mid_first, passes, &wu);
   int write_u = wu ? 1 : 0;
 
   cudaGraph_t g = nullptr;
@@ -1122,7 +1277,7 @@ static int gm_build(const SolvePlan& p, const PcgArgs<TM>& a, cudaGraphExec_t* e
   }
   int nbi = nb_init;
   {
-    void* args[] = {&sc, &bd, &part, &nbi, &h};
+    void* args[] = {&sc, &bd, &part, &nbi, &h, &flags};
     if ((rc = gm_add(g, &prev, reinterpret_cast<const void*>(&k_gm_start), 1, 256, args)) != LAP5CG_OK)
       return fail(rc);
   }
@@ -1139,6 +1294,24 @@ static int gm_build(const SolvePlan& p, const PcgArgs<TM>& a, cudaGraphExec_t* e
     cudaGraphNode_t bp = nullptr;
     Grid<const double> grc{a.r.ptr, a.r.ld};
     for (const GmPassRec<TM>& pr : passes) {
+      if (pr.kind == -2) {
+        const void* fm = reinterpret_cast<const void*>(&k_gm_mid<TM>);
+        if (cudaFuncSetAttribute(fm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem) != cudaSuccess)
+          return fail(LAP5CG_ERR_CUDA);
+        GmLevels<TM> lv;
+        for (int l = 0; l < kMgMaxLevels; ++l) lv.lv[l] = a.lv[l];
+        int nlev = a.nlev, nu_c = a.nu_c;
+        mid.flags = flags;
+        mid.abort_flag = flags + kMidStages * kMidMaxCtas;
+        void* args[] = {&sc, &mid, &lv, &nlev, &mid_small, &nu_c};
+        if ((rc = gm_add(body, &bp, fm, (unsigned)mid_grid, kMidThreads, args, (unsigned)mid_smem)) != LAP5CG_OK)
+          return fail(rc);
+        cudaLaunchAttributeValue coop = {};
+        coop.cooperative = 1;
+        if (cudaGraphKernelNodeSetAttribute(bp, cudaLaunchAttributeCooperative, &coop) != cudaSuccess)
+          return fail(LAP5CG_ERR_CUDA);
+        continue;
+      }
       if (pr.kind < 0) {
         GmLevels<TM> lv;
         for (int l = 0; l < kMgMaxLevels; ++l) lv.lv[l] = a.lv[l];
@@ -1228,24 +1401,15 @@ static int gm_build(const SolvePlan& p, const PcgArgs<TM>& a, cudaGraphExec_t* e
       if ((rc = gm_add(body, &bp, f_pass, (unsigned)grid, kGmThreads, args)) != LAP5CG_OK) return fail(rc);
     }
     int nbp = nb_dot;
-    {
-      void* args[] = {&sc, &part, &nbp};
-      if ((rc = gm_add(body, &bp, reinterpret_cast<const void*>(&k_gm_rz), 1, 256, args)) != LAP5CG_OK)
-        return fail(rc);
-    }
+    double *partq = part + 2 * kGmMaxBlocks, *partx = part;  // the passes' own places
     int zb = zbuf, rev1 = 1, rev0 = 0;
     {
-      void* args[] = {&sc, &bd, &part, &nx_, &ny_, &ld_, &gp0, &gp1, &gq, &L0, &zb, &rev1};
+      void* args[] = {&sc, &bd, &part, &nbp, &partq, &nx_, &ny_, &ld_, &gp0, &gp1, &gq, &L0, &zb, &rev1};
       if ((rc = gm_add(body, &bp, f_pq, nb_pq, kGmThreads, args)) != LAP5CG_OK) return fail(rc);
     }
     int nbq = nb_pq;
     {
-      void* args[] = {&sc, &part, &nbq};
-      if ((rc = gm_add(body, &bp, reinterpret_cast<const void*>(&k_gm_alpha), 1, 256, args)) != LAP5CG_OK)
-        return fail(rc);
-    }
-    {
-      void* args[] = {&sc, &part, &nx_, &ny_, &gr, &gq, &L0, &rev0, &write_u};
+      void* args[] = {&sc, &partq, &nbq, &partx, &nx_, &ny_, &gr, &gq, &L0, &rev0, &write_u};
       if ((rc = gm_add(body, &bp, f_xr, nb_xr, kGmThreads, args)) != LAP5CG_OK) return fail(rc);
     }
     int nbx = nb_xr;
@@ -1303,7 +1467,11 @@ int solve_mg_graph(const SolvePlan& p, const PcgArgs<TM>& a, cudaStream_t st, bo
       break;
     }
   if (!exec) {
-    const int rc = gm_build<TM>(p, a, &exec);
+    int rc = gm_build<TM>(p, a, true, &exec);
+    if (rc != LAP5CG_OK) {  // a driver without cooperative nodes in conditional bodies
+      cudaGetLastError();
+      rc = gm_build<TM>(p, a, false, &exec);
+    }
     if (rc != LAP5CG_OK) {  // a driver without conditional graph nodes: the persistent kernel solves
       cudaGetLastError();
       return LAP5CG_OK;

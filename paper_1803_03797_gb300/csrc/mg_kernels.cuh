@@ -62,6 +62,20 @@ __device__ __forceinline__ double mg_widen(float f) {
 }
 __device__ __forceinline__ double mg_widen(double d) { return d; }
 
+// binary64 -> TM.  binary32: rounding to nearest even on the bits for results in
+// the normal range (the hardware conversion is a slot of the FP64 pipe); others
+// take the hardware conversion.
+template <class TM> __device__ __forceinline__ TM mg_narrow(double d);
+template <> __device__ __forceinline__ double mg_narrow<double>(double d) { return d; }
+template <> __device__ __forceinline__ float mg_narrow<float>(double d) {
+  const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+  const uint32_t e = (hi >> 20) & 0x7ffu;
+  if (e - 897u >= 253u) return (float)d;
+  const uint32_t m = __funnelshift_l(lo, hi & 0x7fffffffu, 3) - (896u << 23), rem = lo << 3;
+  const uint32_t up = (rem > 0x80000000u || (rem == 0x80000000u && (m & 1u))) ? 1u : 0u;
+  return __uint_as_float((m + up) | (hi & 0x80000000u));
+}
+
 // Damped Jacobi sweep (JAC) out = in + c (b - A in), or residual out = b - A in;
 // with DOT also accumulates (r, out) against the binary64 grid r (level 0).
 template <class TM, bool JAC, bool DOT>
