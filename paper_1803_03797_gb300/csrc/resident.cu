@@ -75,6 +75,11 @@ int try_resident(const SolvePlan& p, cudaStream_t st, bool* used) {
   if (rc != LAP5CG_OK) return rc;
   ResPlan g;
   if (!res_plan(kind, p.nx, p.ny, dp.sms, 2, &g)) return LAP5CG_OK;
+  // A wide, flat grid gives rows to few SMs (two rows a CTA at least): past twice the
+  // even share of the items the streaming kernels, which also split columns, are
+  // faster (3000 x 100 binary64: 14.9 against 23.2 us an iteration; 1024 x 24, with 1024
+  // items a CTA, 14.2 against 8.5)
+  if (g.items > 1024 && (long long)g.items * dp.sms > 2 * g.groups * p.ny) return LAP5CG_OK;
   const void* fn = res_kernel_of(kind, g.k);
   if (!fn || g.smem + sizeof(ResShared) + 1024 > (size_t)dp.max_smem_optin) return LAP5CG_OK;
   if (kResSlotOffset + g.slot_bytes > kCtlBytes || kCtlBytes + g.halo_bytes > p.ws_bytes) return LAP5CG_OK;

@@ -18,6 +18,7 @@
 #pragma once
 
 #include "cg_kernels.cuh"
+#include "fixstencil.cuh"
 
 namespace lap5 {
 
@@ -263,27 +264,52 @@ struct ResItems {
   }
 };
 
-// y = A c on item k from the shared rows sm (c: the item itself), in the order
-// 4C - W - E - S - N.  up / dn: rows above / below.  Whole-warp call.
+// y = A c on item k from the shared rows sm (c: the item itself; up / dn: rows above
+// / below), binary32 in the order 4C - W - E - S - N, binary64 in fixed point
+// (fixstencil.cuh; one FP64 operation a point instead of four).  Whole-warp call.
 template <class T, int K, class M>
 __device__ __forceinline__ void res_stencil(const ResItems<T, K>& it, int k, const T* sm, const M (&c)[ResVec<T>::W],
                                             const M (&up)[ResVec<T>::W], const M (&dn)[ResVec<T>::W],
                                             M (&y)[ResVec<T>::W]) {
   constexpr int W = ResVec<T>::W;
   const int lane = threadIdx.x & 31, o = it.off[k];
-  M l = shfl_up1(c[W - 1]), r = shfl_dn1(c[0]);
-  if (it.is(it.first, k)) l = M(0);
-  else if (lane == 0) l = (M)sm[o - 1];
-  if (it.is(it.last, k)) r = M(0);
-  else if (lane == 31) r = (M)sm[o + W];
+  const bool lh = lane == 0 && !it.is(it.first, k), rh = lane == 31 && !it.is(it.last, k);
+  if constexpr (sizeof(T) == 8) {
+    double h = 0.0;  // the column beyond the warp's first or last item
+    if (lh) h = sm[o - 1];
+    if (rh) h = sm[o + W];
+    unsigned m = fix_mag(h);
 #pragma unroll
-  for (int q = 0; q < W; ++q) {
-    M a = M(4) * c[q];
-    a -= q == 0 ? l : c[q - 1];
-    a -= q == W - 1 ? r : c[q + 1];
-    a -= up[q];
-    a -= dn[q];
-    y[q] = a;
+    for (int q = 0; q < W; ++q) m = max(max(m, fix_mag(c[q])), max(fix_mag(up[q]), fix_mag(dn[q])));
+    const int E = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
+    long long f[W], s[W];
+#pragma unroll
+    for (int q = 0; q < W; ++q) f[q] = fix_of(c[q], E);
+    const long long e = fix_of(h, E);
+    long long l = __shfl_up_sync(0xffffffffu, f[W - 1], 1), r = __shfl_down_sync(0xffffffffu, f[0], 1);
+    if (it.is(it.first, k)) l = 0;
+    else if (lane == 0) l = e;
+    if (it.is(it.last, k)) r = 0;
+    else if (lane == 31) r = e;
+#pragma unroll
+    for (int q = 0; q < W; ++q)
+      s[q] = 4 * f[q] - (q == 0 ? l : f[q - 1]) - (q == W - 1 ? r : f[q + 1]) - fix_of(up[q], E) - fix_of(dn[q], E);
+    fix_results<W>(s, E, y);
+  } else {
+    M l = shfl_up1(c[W - 1]), r = shfl_dn1(c[0]);
+    if (it.is(it.first, k)) l = M(0);
+    else if (lh) l = (M)sm[o - 1];
+    if (it.is(it.last, k)) r = M(0);
+    else if (rh) r = (M)sm[o + W];
+#pragma unroll
+    for (int q = 0; q < W; ++q) {
+      M a = M(4) * c[q];
+      a -= q == 0 ? l : c[q - 1];
+      a -= q == W - 1 ? r : c[q + 1];
+      a -= up[q];
+      a -= dn[q];
+      y[q] = a;
+    }
   }
   it.mask_tail(k, y);
 }
