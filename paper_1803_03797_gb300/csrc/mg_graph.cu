@@ -685,8 +685,7 @@ __global__ void __launch_bounds__(kMidThreads, 1) k_gm_mid(GmScal* sc, MidArgs<T
     mid_signal(flags(n + 1), tag);
     return;
   }
-  for (size_t i = threadIdx.x; i < (size_t)m.offE; i += blockDim.x) sm[i] = TM(0);  // pads stay zero
-  __syncthreads();
+  for (int l = 0; l < n; ++l) mid_zero_pads<TM>(m.lv[l], sm);
   auto below = [&](int l) -> const MgLevel<TM>& { return l + 1 < n ? m.lv[l + 1].g : levels.lv[small_first]; };
   for (int l = 0; l < n; ++l) {
     const MidLevel<TM>& L = m.lv[l];

@@ -171,6 +171,18 @@ __device__ __forceinline__ void mid_signal(int* flag, int tag) {
   }
 }
 
+// The columns before and after the vectors of a level's rows, zero for good (the next
+// CTA barrier publishes them).
+template <class TM>
+__device__ __forceinline__ void mid_zero_pads(const MidLevel<TM>& L, TM* sm) {
+  constexpr int W = MidVec<TM>::W;
+  const int used = (L.g.nx + W - 1) / W * W, rows = 2 * L.R + 10, pads = L.ldp - used;  // b and u rows are adjacent
+  for (int i = threadIdx.x; i < rows * pads; i += blockDim.x) {
+    const int r = i / pads, k = i - r * pads;
+    sm[L.offB + r * L.ldp + (k < 4 ? k : used + k)] = TM(0);
+  }
+}
+
 // Down one level: loads b, forms u (kept), restricts the residual.
 template <class TM>
 __device__ __forceinline__ void mid_down(const MidLevel<TM>& L, const MgLevel<TM>& C, TM* sm, int offT, int cta) {
