@@ -5,8 +5,8 @@
 // (addition) cycles on each scheduler, the integer pipe one a cycle.  The four FP64
 // operations a point of the mask are 292 cycles of the pipe that bounds the
 // binary64 CG passes; in fixed point they are about 45 integer instructions and
-// one conversion back (64).  4096^2, an iteration: classic 302 -> 222 us, NewCG 375 ->
-// 311 us.
+// one conversion back (64; the ring kernels do that in integers too, 48).  4096^2, an
+// iteration, by itself: classic 302 -> 222 us, NewCG 375 -> 311 us.
 //
 // How: a row's values are aligned to the largest exponent among the warp's values
 // of the row (one redux.sync), as signed multiples of 2^-58 of that exponent's
@@ -50,6 +50,23 @@ __device__ __forceinline__ double fix_to(long long q, int E) {
   const double v = (double)q;
   const int hi = __double2hiint(v);
   return __hiloint2double(hi == 0 ? 0 : hi + ((E - kFixBias) << 20), __double2loint(v));
+}
+
+// The same on the integer pipe (about 40 instructions; the conversion above is one
+// slot of the FP64 pipe, 64 cycles), |q| < 2^63: the magnitude with its leading bit
+// moved to bit 62 (nothing lost), rounded to 53 bits half to even, the carry running
+// into the exponent field.  For the ring kernels, which the FP64 pipe bounds (80-85 %
+// busy) at half the issue slots: 4096^2, classic 211 -> 195 us an iteration, NewCG 302
+// -> 288.  The resident and multigrid kernels, whose warps wait on a chain rather than
+// on the pipe, are faster with the conversion (1024^2 f64 20.5 against 20.9 us).
+__device__ __forceinline__ double fix_to_int(long long q, int E) {
+  const unsigned long long s = (unsigned long long)(q >> 63), a = ((unsigned long long)q ^ s) - s;
+  const int lz = __clzll((long long)a);
+  const unsigned long long t = a << ((lz - 1) & 63);
+  const unsigned long long m = (t + 0x1ffull + ((t >> 10) & 1ull)) >> 10;
+  unsigned long long b = m + ((unsigned long long)(unsigned)(E + 4 - lz) << 52);
+  if (a == 0ull) b = 0ull;
+  return __longlong_as_double((long long)(b | (s << 63)));
 }
 
 // One row of a strip: the lane's V values at the row's exponent.
@@ -113,7 +130,7 @@ __device__ __forceinline__ void march_ring_fix(WarpRing& ring, int ny, int lane,
       fix_align<V>(n, a.E, E);
       double y[V];
 #pragma unroll
-      for (int k = 0; k < V; ++k) y[k] = fix_to(sum.q[k] - n[k], E);
+      for (int k = 0; k < V; ++k) y[k] = fix_to_int(sum.q[k] - n[k], E);
       if (E < kFixLow || E > kFixHigh) {
 #pragma unroll
         for (int k = 0; k < V; ++k) y[k] = E < kFixLow ? 0.0 : __longlong_as_double(0x7ff8000000000000ll);
