@@ -138,7 +138,8 @@ int solve_typed(const SolvePlan& plan, cudaStream_t st) {
     }
     rc = plan_units(fn, p.nx, p.ny, V, p.opts, dyn, &cfg, row_align);
     if (rc != LAP5CG_OK) return rc;
-    if (ring && p.opts.ring_slots == 0 && cfg.seg_rows < kRingMinRows) {  // short units: register march
+    if (ring && p.opts.ring_slots == 0 &&
+        cfg.seg_rows < ring_min_rows(RingOnly<T, V>::value, p.opts)) {  // short units: register march
       if constexpr (RingOnly<T, V>::value) {
         return LAP5CG_ERR_UNSUPPORTED;  // the caller narrows the lane vector
       } else {

@@ -57,7 +57,7 @@ static int solve_ir_t(const SolvePlan& plan, cudaStream_t st) {
   }
   rc = plan_units(fn, p.nx, p.ny, V, p.opts, dyn, &cfg);
   if (rc != LAP5CG_OK) return rc;
-  if (ring && p.opts.ring_slots == 0 && cfg.seg_rows < kRingMinRows) {  // short units: register march
+  if (ring && p.opts.ring_slots == 0 && cfg.seg_rows < ring_min_rows(Lanes<V>::G > 1, p.opts)) {  // short units: register march
     if constexpr (Lanes<V>::G > 1) {
       return LAP5CG_ERR_UNSUPPORTED;  // the caller narrows the lane vector
     } else {

@@ -137,6 +137,19 @@ constexpr int kDefaultMinRows = 2;        // shortest warp unit (rows) on small 
 constexpr int kRingBytesPerWarp = 12800;  // 16 warps per SM fit 228 KB of shared memory
 constexpr int kRingMinRows = 8;           // automatic ring only for units at least this tall
 
+// Wide lanes (eight binary32 columns, four binary64) are only built with the
+// ring; half as many columns mean twice the row steps a point.  Chosen by the
+// library (not by lane_vec) they are worth it from units of five rows on, where
+// the narrow choice has eight and a ring too (us an iteration, narrow -> wide:
+// binary32 classic 2048^2, 7 rows, 32.6 -> 26.3; 1600^2, 5 rows, 25.0 -> 21.3;
+// IR_F32 1600^2 26.8 -> 21.7; binary64 classic 1300^2, 6 rows, 38.4 -> 33.0; 1100^2,
+// 5 rows, 31.7 -> 29.7).  At four rows the narrow register march can be the faster
+// (IR_F32 1300^2 17.5 against 19.3).
+constexpr int kRingMinRowsWide = 5;
+inline int ring_min_rows(bool wide, const lap5cg_opts& o) {
+  return wide && o.lane_vec == 0 ? kRingMinRowsWide : kRingMinRows;
+}
+
 constexpr size_t kCtlBytes = 256 * 1024;  // control block region at the workspace start
 constexpr size_t kAlign = 256;
 __host__ __device__ inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
