@@ -1,7 +1,9 @@
 // batched.cu -- cg_solve_batched: many independent grids of different shapes
 // in one persistent launch.
 //
-// A team is one thread-block cluster (1, 2, 4, 8 or 16 CTAs).  Teams pull the
+// Instances whose state fits in the SMs of a team go to the chip-resident
+// kernels first (resident.cu; a launch or a few for all of them); what follows
+// is for the rest.  A team is one thread-block cluster (1, 2, 4, 8 or 16 CTAs).  Teams pull the
 // next instance from an atomic queue over a table sorted by estimated work
 // (largest first: grid points x (nx + ny), since CG iterations grow with the
 // side length), solve it with the same fused passes as the single-grid
