@@ -224,6 +224,14 @@ __device__ __forceinline__ Acc make_acc(Team& tm, int slot, int ny, bool rev) {
   return a;
 }
 
+// The barrier of an exact reduction, as a call (the epoch by value): inlined, its
+// registers made the row march of the reproducible NewCG spill.
+template <class C>
+__device__ __noinline__ bool exact_barrier(C* ctl, unsigned long long epoch, double* red, long long timeout_ns) {
+  double v[1] = {0.0}, o[1];
+  return grid_reduce<1>(ctl, epoch, v, o, red, timeout_ns);
+}
+
 // Exact reduction of the NV dot products accumulated in the CTAs' shared
 // accumulators (slots 0..NV-1): every CTA adds its accumulators into the
 // solve's global accumulator of this reduction, the grid barrier, then every
@@ -252,8 +260,8 @@ __device__ __forceinline__ bool grid_reduce_exact(GridTeam& tm, double (&out)[NV
     if (threadIdx.x < kExactSlots) ctl->xbad[en][threadIdx.x] = 0u;
   }
   ++tm.xepoch;
-  double v[1] = {0.0}, o[1];
-  if (!grid_reduce<1>(ctl, tm.epoch, v, o, red, tm.timeout_ns)) return false;
+  const unsigned long long epoch = tm.epoch++;
+  if (!exact_barrier(ctl, epoch, red, tm.timeout_ns)) return false;
   // the totals, read past L1 (other SMs' atomics landed in L2); the CTA's own
   // accumulators are zero again and serve as scratch
   for (int t = threadIdx.x; t < NV * kExactLimbs; t += blockDim.x)
