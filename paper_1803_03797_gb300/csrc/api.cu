@@ -28,6 +28,19 @@ int dev_props(DevProps* out) {
   return LAP5CG_OK;
 }
 
+int allow_dyn_smem(const void* fn, size_t bytes) {
+  DevProps dp;
+  const int rc = dev_props(&dp);
+  if (rc != LAP5CG_OK) return rc;
+  cudaFuncAttributes fa;
+  if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) return LAP5CG_ERR_CUDA;
+  const int most = dp.max_smem_optin - (int)fa.sharedSizeBytes;
+  if (most < 0 || bytes > (size_t)most) return LAP5CG_ERR_CUDA;
+  if (fa.maxDynamicSharedSizeBytes >= most) return LAP5CG_OK;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess ? LAP5CG_OK
+                                                                                                    : LAP5CG_ERR_CUDA;
+}
+
 int warps_of(const lap5cg_opts& o) {
   int wpc = o.warps_per_cta > 0 ? o.warps_per_cta : kDefaultWarps;
   return wpc > 16 ? 16 : wpc;
@@ -101,8 +114,7 @@ int choose_ring(const void* func, int slot_bytes, const lap5cg_opts& o, int wpc,
     if (o.ring_slots > 0) return LAP5CG_ERR_UNSUPPORTED;
     return LAP5CG_OK;
   }
-  if (cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-    return LAP5CG_ERR_CUDA;
+  if ((rc = allow_dyn_smem(func, dyn)) != LAP5CG_OK) return rc;
   g->S = S;
   g->warp_bytes = warp_bytes;
   *dyn_smem = dyn;

@@ -98,6 +98,12 @@ struct DevProps {
 };
 int dev_props(DevProps* out);
 
+// Lets launches of fn use `bytes` of dynamic shared memory.  The limit belongs to the
+// function, not to a launch, so every call sets the same value (all that fn's static
+// shared memory leaves): a size of its own would lower the limit under a launch of
+// another thread, or under graph nodes recorded with more.
+int allow_dyn_smem(const void* fn, size_t bytes);
+
 // Grid sizing shared by the persistent kernels: fills cfg from the occupancy
 // of kernel func at the requested warps per CTA.
 int plan_units(const void* func, int nx, int ny, int V, const lap5cg_opts& o, size_t dyn_smem, LaunchCfg* cfg,

@@ -1295,8 +1295,7 @@ static int gm_build(const SolvePlan& p, const PcgArgs<TM>& a, bool use_mid, cuda
     for (const GmPassRec<TM>& pr : passes) {
       if (pr.kind == -2) {
         const void* fm = reinterpret_cast<const void*>(&k_gm_mid<TM>);
-        if (cudaFuncSetAttribute(fm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mid_smem) != cudaSuccess)
-          return fail(LAP5CG_ERR_CUDA);
+        if ((rc = allow_dyn_smem(fm, mid_smem)) != LAP5CG_OK) return fail(rc);
         GmLevels<TM> lv;
         for (int l = 0; l < kMgMaxLevels; ++l) lv.lv[l] = a.lv[l];
         int nlev = a.nlev, nu_c = a.nu_c;
@@ -1322,8 +1321,7 @@ static int gm_build(const SolvePlan& p, const PcgArgs<TM>& a, bool use_mid, cuda
         cudaFuncAttributes fa;
         if (cudaFuncGetAttributes(&fa, fs) != cudaSuccess) return fail(LAP5CG_ERR_CUDA);
         if (smem + fa.sharedSizeBytes <= (size_t)dp.max_smem_optin) {
-          if (cudaFuncSetAttribute(fs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return fail(LAP5CG_ERR_CUDA);
+          if ((rc = allow_dyn_smem(fs, smem)) != LAP5CG_OK) return fail(rc);
         } else {
           fs = reinterpret_cast<const void*>(&k_gm_small<TM, false>);
           smem = 0;

@@ -84,8 +84,8 @@ int try_resident(const SolvePlan& p, cudaStream_t st, bool* used) {
   if (!fn || g.smem + sizeof(ResShared) + 1024 > (size_t)dp.max_smem_optin) return LAP5CG_OK;
   if (kResSlotOffset + g.slot_bytes > kCtlBytes || kCtlBytes + g.halo_bytes > p.ws_bytes) return LAP5CG_OK;
   if (g.smem + sizeof(ResShared) > 48 * 1024 &&  // beyond the size every launch may use
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem) != cudaSuccess)
-    return LAP5CG_ERR_CUDA;
+      (rc = allow_dyn_smem(fn, g.smem)) != LAP5CG_OK)
+    return rc;
   // tags of an earlier solve in this workspace must not be taken for this one's
   if (cudaMemsetAsync(p.ws, 0, kResSlotOffset + g.slot_bytes, st) != cudaSuccess ||
       cudaMemsetAsync(p.ws + kCtlBytes, 0, g.halo_bytes, st) != cudaSuccess)
@@ -160,9 +160,10 @@ static double res_makespan(int kind, const std::vector<ResPick>& v, const int* n
 }
 
 static int res_launch_batch(const void* fn, ResBatchLaunch l, int teams, size_t smem, cudaStream_t st) {
-  if (smem + sizeof(ResShared) > 48 * 1024 - 64 &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return LAP5CG_ERR_CUDA;
+  if (smem + sizeof(ResShared) > 48 * 1024 - 64) {
+    const int rc = allow_dyn_smem(fn, smem);
+    if (rc != LAP5CG_OK) return rc;
+  }
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(teams * l.team);
   lc.blockDim = dim3(kResMaxThreads);

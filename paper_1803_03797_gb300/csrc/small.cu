@@ -598,8 +598,7 @@ static int try_small_t(const SolvePlan& p, cudaStream_t st, bool* used) {
   const size_t smem = small_smem<T>(p.nx, p.ny, p.variant, C, &R, &ldp);
   if (smem + sizeof(double) * kRedDoubles + 1024 > (size_t)dp.max_smem_optin) return LAP5CG_OK;  // too large
   const void* fn = reinterpret_cast<const void*>(&k_small<T>);
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return LAP5CG_ERR_CUDA;
+  if ((rc = allow_dyn_smem(fn, smem)) != LAP5CG_OK) return rc;
   if (C > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
     return LAP5CG_ERR_CUDA;
   SmallArgs<T> a;
@@ -682,8 +681,7 @@ static int small_batched_t(int count, const int* nx, const int* ny, const int* l
   }
   if (pick.empty()) return LAP5CG_OK;
   const void* fn = reinterpret_cast<const void*>(&k_small_batch<T>);
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max) != cudaSuccess)
-    return LAP5CG_ERR_CUDA;
+  if ((rc = allow_dyn_smem(fn, smem_max)) != LAP5CG_OK) return rc;
   if (C > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
     return LAP5CG_ERR_CUDA;
   cudaLaunchConfig_t lc = {};
