@@ -41,7 +41,14 @@ struct GmScal {
   double bb, thr, rr, gamma[2], alpha;  // gamma: by iteration parity
   int iters, status, stop, cur, zero_x;
   int xpend;  // x += alpha p of the last x, r pass is still to be applied (k_gm_pq or k_gm_xfinal)
+  // An iteration that cannot go on, by the pass that found it (GM_BAD_*).  stop is tested on
+  // entry by every thread of a pass, so only one-CTA kernels write it: set by a CTA of
+  // a running launch, it would send some warps of a late CTA home and leave the others
+  // to sum without them.  A pass tests the words of earlier passes only; k_gm_check
+  // turns any of them into stop.
+  int bad[3];
 };
+enum { GM_BAD_MID = 0, GM_BAD_PQ, GM_BAD_XR };
 
 // Per-call arguments, written by k_gm_bind before each graph launch, so that
 // one instantiated graph serves every right-hand side, solution, tolerance and
@@ -673,7 +680,7 @@ __global__ void __launch_bounds__(kMidThreads, 1) k_gm_mid(GmScal* sc, MidArgs<T
   auto fail = [&]() {
     if (threadIdx.x == 0) {
       sc->status = LAP5CG_ERR_SYNC_TIMEOUT;
-      sc->stop = 1;
+      sc->bad[GM_BAD_MID] = 1;
     }
   };
   // stages: [1, n] b of distributed level 1 .. n - 1 and of the small levels
@@ -849,7 +856,7 @@ __global__ void __launch_bounds__(kGmThreads) k_gm_pq(GmScal* sc, const GmBind* 
                                                        double* part, int nx, int ny, int ld, Grid<double> p0,
                                                        Grid<double> p1, Grid<double> q, MgLevel<TM> L0, int zbuf,
                                                        int rev) {
-  if (sc->stop) return;
+  if (sc->stop || sc->bad[GM_BAD_MID]) return;
   constexpr int V = 2;
   const Sched s = gm_sched(rev);
   const Units un = make_units(nx, ny, V, s.nw, 2);
@@ -861,7 +868,7 @@ __global__ void __launch_bounds__(kGmThreads) k_gm_pq(GmScal* sc, const GmBind* 
     if (!bits_positive(rz) || !bits_finite(rz)) {  // (the same in every CTA)
       if (blockIdx.x == 0 && threadIdx.x == 0) {
         sc->status = LAP5CG_ERR_BREAKDOWN;
-        sc->stop = 1;
+        sc->bad[GM_BAD_PQ] = 1;
       }
       return;
     }
@@ -935,7 +942,7 @@ __global__ void __launch_bounds__(kGmThreads) k_gm_xr(GmScal* sc, const double* 
                                                        int ny,
                                                        Grid<double> r, Grid<double> q, MgLevel<TM> L0, int rev,
                                                        int write_u) {
-  if (sc->stop) return;
+  if (sc->stop || sc->bad[GM_BAD_MID] || sc->bad[GM_BAD_PQ]) return;
   constexpr int V = 2;
   const Sched s = gm_sched(rev);
   const Units un = make_units(nx, ny, V, s.nw, 2);
@@ -953,7 +960,7 @@ __global__ void __launch_bounds__(kGmThreads) k_gm_xr(GmScal* sc, const double* 
           sc->cur ^= 1;
         } else {
           sc->status = LAP5CG_ERR_BREAKDOWN;
-          sc->stop = 1;
+          sc->bad[GM_BAD_XR] = 1;
         }
       }
     }
@@ -997,8 +1004,11 @@ __global__ void __launch_bounds__(kGmThreads) k_gm_xr(GmScal* sc, const double* 
 // (r, r) -> iteration count, history, convergence; the loop's condition.
 __global__ void __launch_bounds__(256) k_gm_check(GmScal* sc, const GmBind* bd, const double* part, int nb,
                                                   cudaGraphConditionalHandle h) {
-  if (sc->stop) {
-    if (threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
+  if (sc->bad[GM_BAD_MID] || sc->bad[GM_BAD_PQ] || sc->bad[GM_BAD_XR]) {
+    if (threadIdx.x == 0) {
+      sc->stop = 1;
+      cudaGraphSetConditional(h, 0u);
+    }
     return;
   }
   const double rr = gm_total(part, nb, 0);
