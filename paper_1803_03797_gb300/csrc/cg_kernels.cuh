@@ -269,7 +269,7 @@ __device__ void classic_solve(const ClassicArgs<T>& a, Team& tm, double* red, un
             };
             if constexpr (FIX) {
               auto finish = [&](int j, const unsigned char*, const M (&p)[V], const M (&ap)[V]) { row(j, p, ap); };
-              march_ring_fix<V>(ring, c.ny, wk.lane, xs, y0, y1, wk.rev(), vv, off, field, finish);
+              march_ring_fix<V>(ring, c.ny, wk.lane, xs, nval, y0, y1, wk.rev(), vv, off, field, finish);
             } else {
               auto finish = [&](int j, const unsigned char*, const FRow<V, M>& S, const FRow<V, M>& C,
                                 const FRow<V, M>& N) {
@@ -733,7 +733,7 @@ __device__ void newcg_solve(const NewcgArgs<T>& a, Team& tm, double* red, unsign
             store_row<V>(wn, j, xl, c.nx, wv);
           };
           if constexpr (FIX) {
-            march_ring_fix<V>(ring, c.ny, wk.lane, xs, y0, y1, wk.rev(), vv, off, field, row);
+            march_ring_fix<V>(ring, c.ny, wk.lane, xs, nval, y0, y1, wk.rev(), vv, off, field, row);
           } else {
             auto finish = [&](int j, const unsigned char* sl, const FRow<V, M>& S, const FRow<V, M>& C,
                               const FRow<V, M>& N) {

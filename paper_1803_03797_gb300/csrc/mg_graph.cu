@@ -182,41 +182,52 @@ __global__ void __launch_bounds__(kGmThreads) k_gm_sweep(const GmScal* sc, doubl
       }
     }
     TM rs[R][V];  // b - A u
+    bool fixed = false;
     if constexpr (sizeof(TM) == 8) {
       // binary64: in fixed point over the tile's rows (fixstencil.cuh), one FP64
       // operation a point instead of five
-      unsigned m = 0u;
+      static_assert(V == 2, "a point's row neighbour in the lane");
+      unsigned m = 0u, n = 0x7fffffffu;
 #pragma unroll
       for (int k = 0; k < R + 2; ++k) {
 #pragma unroll
         for (int q = 0; q < V; ++q) m = max(m, fix_mag(f[k].f[q]));
         if (k >= 1 && k <= R) {
           m = max(m, max(fix_mag(f[k].hl), fix_mag(f[k].hr)));
+          const unsigned cc = max(fix_mag(f[k].f[0]), fix_mag(f[k].f[1]));
 #pragma unroll
-          for (int q = 0; q < V; ++q) m = max(m, fix_mag(bv[k - 1][q]));
+          for (int q = 0; q < V; ++q) {
+            m = max(m, fix_mag(bv[k - 1][q]));
+            const unsigned p = max(cc, max(fix_mag(f[k - 1].f[q]), fix_mag(f[k + 1].f[q])));
+            if (jb + k - 1 < L.ny && xl + q < L.nx) n = min(n, p);
+          }
         }
       }
       const int E = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
-      long long w[R + 2][V];
+      fixed = fix_fits<kFixSpanRes>(n, E);
+      if (fixed) {
+        long long w[R + 2][V];
 #pragma unroll
-      for (int k = 0; k < R + 2; ++k)
+        for (int k = 0; k < R + 2; ++k)
 #pragma unroll
-        for (int q = 0; q < V; ++q) w[k][q] = fix_of(f[k].f[q], E);
+          for (int q = 0; q < V; ++q) w[k][q] = fix_of<kFixBRes>(f[k].f[q], E);
 #pragma unroll
-      for (int k = 0; k < R; ++k) {
-        const long long h = fix_of(lane == 0 ? f[k + 1].hl : f[k + 1].hr, E);
-        long long l = __shfl_up_sync(0xffffffffu, w[k + 1][V - 1], 1);
-        long long r = __shfl_down_sync(0xffffffffu, w[k + 1][0], 1);
-        if (lane == 0) l = h;
-        if (lane == 31) r = h;
-        long long d[V];
+        for (int k = 0; k < R; ++k) {
+          const long long h = fix_of<kFixBRes>(lane == 0 ? f[k + 1].hl : f[k + 1].hr, E);
+          long long l = __shfl_up_sync(0xffffffffu, w[k + 1][V - 1], 1);
+          long long r = __shfl_down_sync(0xffffffffu, w[k + 1][0], 1);
+          if (lane == 0) l = h;
+          if (lane == 31) r = h;
 #pragma unroll
-        for (int q = 0; q < V; ++q)
-          d[q] = fix_of(bv[k][q], E) - 4 * w[k + 1][q] + (q == 0 ? l : w[k + 1][q - 1]) +
-                 (q == V - 1 ? r : w[k + 1][q + 1]) + w[k][q] + w[k + 2][q];
-        fix_results<V>(d, E, rs[k]);
+          for (int q = 0; q < V; ++q)
+            rs[k][q] = fix_to<kFixBRes>(fix_of<kFixBRes>(bv[k][q], E) - 4 * w[k + 1][q] +
+                                            (q == 0 ? l : w[k + 1][q - 1]) + (q == V - 1 ? r : w[k + 1][q + 1]) +
+                                            w[k][q] + w[k + 2][q],
+                                        E);
+        }
       }
-    } else {
+    }
+    if (!fixed) {
 #pragma unroll
       for (int k = 0; k < R; ++k) {
         TM ax[V];
@@ -927,7 +938,7 @@ __global__ void __launch_bounds__(kGmThreads) k_gm_pq(GmScal* sc, const GmBind* 
       store_row<V>(q, j, xl, nx, qv);
       acc_dot<V>(apq, j, pv, qv, nval);
     };
-    march_fix<V, Raw>(ny, s.lane, y0, y1, s.rev, load, field, finish);
+    march_fix<V, Raw>(ny, s.lane, nval, y0, y1, s.rev, load, field, finish);
   }
   const double v[1] = {apq.value()};
   gm_partials<1>(v, part);

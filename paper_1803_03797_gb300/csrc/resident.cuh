@@ -14,7 +14,10 @@
 //
 // Arithmetic per point is that of the streaming kernels (Algorithm 1 with
 // z = A p stored and the x update deferred to the next direction update;
-// Algorithm 2); dot products differ in summation order only.
+// Algorithm 2).  The sums of dot products differ in order, and binary64 stencils in
+// rounding: fixed point (fixstencil.cuh) aligned to the largest value of a warp's items,
+// which may lie in several rows, where the row-ring kernels align a strip's rows
+// and the register marches add in FP64.
 #pragma once
 
 #include "cg_kernels.cuh"
@@ -278,23 +281,43 @@ __device__ __forceinline__ void res_stencil(const ResItems<T, K>& it, int k, con
     double h = 0.0;  // the column beyond the warp's first or last item
     if (lh) h = sm[o - 1];
     if (rh) h = sm[o + W];
-    unsigned m = fix_mag(h);
+    unsigned m = fix_mag(h), n = 0x7fffffffu;
+    const unsigned cc = max(fix_mag(c[0]), fix_mag(c[1]));
 #pragma unroll
-    for (int q = 0; q < W; ++q) m = max(max(m, fix_mag(c[q])), max(fix_mag(up[q]), fix_mag(dn[q])));
+    for (int q = 0; q < W; ++q) {
+      const unsigned p = max(cc, max(fix_mag(up[q]), fix_mag(dn[q])));
+      m = max(m, p);
+      if (it.is(it.valid, k) && !(q > 0 && it.tail < W && it.is(it.last, k))) n = min(n, p);
+    }
     const int E = (int)(__reduce_max_sync(0xffffffffu, m) >> 20);
-    long long f[W], s[W];
+    if (fix_fits<kFixSpan>(n, E)) {
+      long long f[W];
 #pragma unroll
-    for (int q = 0; q < W; ++q) f[q] = fix_of(c[q], E);
-    const long long e = fix_of(h, E);
-    long long l = __shfl_up_sync(0xffffffffu, f[W - 1], 1), r = __shfl_down_sync(0xffffffffu, f[0], 1);
-    if (it.is(it.first, k)) l = 0;
-    else if (lane == 0) l = e;
-    if (it.is(it.last, k)) r = 0;
-    else if (lane == 31) r = e;
+      for (int q = 0; q < W; ++q) f[q] = fix_of<kFixB>(c[q], E);
+      const long long e = fix_of<kFixB>(h, E);
+      long long l = __shfl_up_sync(0xffffffffu, f[W - 1], 1), r = __shfl_down_sync(0xffffffffu, f[0], 1);
+      if (it.is(it.first, k)) l = 0;
+      else if (lane == 0) l = e;
+      if (it.is(it.last, k)) r = 0;
+      else if (lane == 31) r = e;
 #pragma unroll
-    for (int q = 0; q < W; ++q)
-      s[q] = 4 * f[q] - (q == 0 ? l : f[q - 1]) - (q == W - 1 ? r : f[q + 1]) - fix_of(up[q], E) - fix_of(dn[q], E);
-    fix_results<W>(s, E, y);
+      for (int q = 0; q < W; ++q)
+        y[q] = fix_to<kFixB>(4 * f[q] - (q == 0 ? l : f[q - 1]) - (q == W - 1 ? r : f[q + 1]) -
+                                 fix_of<kFixB>(up[q], E) - fix_of<kFixB>(dn[q], E),
+                             E);
+    } else {
+      double l = shfl_up1(c[W - 1]), r = shfl_dn1(c[0]);
+      if (it.is(it.first, k)) l = 0.0;
+      else if (lane == 0) l = h;
+      if (it.is(it.last, k)) r = 0.0;
+      else if (lane == 31) r = h;
+#pragma unroll
+      for (int q = 0; q < W; ++q) {
+        double a = __fma_rn(4.0, c[q], -(q == 0 ? l : c[q - 1]));
+        a = __dsub_rn(a, q == W - 1 ? r : c[q + 1]);
+        y[q] = __dsub_rn(__dsub_rn(a, up[q]), dn[q]);
+      }
+    }
   } else {
     M l = shfl_up1(c[W - 1]), r = shfl_dn1(c[0]);
     if (it.is(it.first, k)) l = M(0);
