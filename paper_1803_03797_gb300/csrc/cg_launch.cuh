@@ -115,7 +115,8 @@ struct RingOnly {
 template <class T, int V, bool EX = false>
 int solve_typed(const SolvePlan& plan, cudaStream_t st) {
   SolvePlan p = plan;
-  p.opts = with_warps(plan.opts, plan.variant == LAP5CG_CLASSIC ? ring_slot_classic(V, (int)sizeof(T))
+  if (EX && p.opts.warps_per_cta == 0) p.opts.warps_per_cta = kExactWarps;
+  p.opts = with_warps(p.opts, plan.variant == LAP5CG_CLASSIC ? ring_slot_classic(V, (int)sizeof(T))
                                                                 : ring_slot_newcg(V, (int)sizeof(T)));
   const size_t vec = align_up((size_t)p.ny * (size_t)p.ldw * sizeof(T), kAlign);
   unsigned char* base = p.ws + kCtlBytes;

@@ -389,7 +389,7 @@ struct Ctl {
   // buffers used in turn by successive exact reductions
   unsigned long long xacc[3][kExactSlots][kExactLimbs];
   unsigned xbad[3][kExactSlots];
-  unsigned xpad[2];
+  unsigned long long xbar;             // arrivals at the exact reductions' barrier
   // per-CTA partials, double-buffered by barrier parity; launches of at most
   // kMaxPeers CTAs exchange them as messages here (slots of kSlotWords words)
   double part[2][kMaxCtas][kMaxVals];

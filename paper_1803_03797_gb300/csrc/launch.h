@@ -139,6 +139,10 @@ inline int ring_slot_ir(int V, int es_r) {
 
 // Launch defaults (measured on GB300; the autotuner can override them).
 constexpr int kDefaultWarps = 16;         // warps per CTA: one CTA an SM, the reductions' peers
+// The same in the reproducible mode, whose warps add blocks to accumulators that their CTA
+// shares (us an iteration with 4 and 16 warps: classic 100^2 41 and 56, 500^2 41 and
+// 67, 1500^2 68 and 68; NewCG 100^2 48 and 66, 500^2 48 and 79, 4096^2 449 and 449).
+constexpr int kExactWarps = 4;
 constexpr int kDefaultMinRows = 2;        // shortest warp unit (rows) on small grids
 constexpr int kRingBytesPerWarp = 12800;  // 16 warps per SM fit 228 KB of shared memory
 constexpr int kRingMinRows = 8;           // automatic ring only for units at least this tall

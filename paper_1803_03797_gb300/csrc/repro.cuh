@@ -224,12 +224,36 @@ __device__ __forceinline__ Acc make_acc(Team& tm, int slot, int ny, bool rev) {
   return a;
 }
 
-// The barrier of an exact reduction, as a call (the epoch by value): inlined, its
-// registers made the row march of the reproducible NewCG spill.
-template <class C>
-__device__ __noinline__ bool exact_barrier(C* ctl, unsigned long long epoch, double* red, long long timeout_ns) {
-  double v[1] = {0.0}, o[1];
-  return grid_reduce<1>(ctl, epoch, v, o, red, timeout_ns);
+// The barrier of the n-th exact reduction (from 1), with a counter of its own: the
+// values travel through the accumulators, and the registers of a message exchange
+// made the row march of the reproducible NewCG spill.  Every thread calls; false when the
+// solve must stop.
+__device__ __forceinline__ bool exact_barrier(Ctl* ctl, unsigned n, long long timeout_ns) {
+  __shared__ int s_xgo;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int go = 1;
+    __threadfence();
+    atomicAdd(&ctl->xbar, 1ull);
+    const unsigned long long target = (unsigned long long)n * gridDim.x;
+    const unsigned long long t0 = global_ns();
+    unsigned spins = 0;
+    while (ld_acquire_u64(&ctl->xbar) < target) {
+      if ((++spins & 7u) == 0u) {  // each poll is an L2 round trip: check the clock often
+        if (ld_relaxed_i32(&ctl->abort)) { go = 0; break; }
+        if ((long long)(global_ns() - t0) > timeout_ns) {
+          record_error(ctl, LAP5CG_ERR_SYNC_TIMEOUT);
+          go = 0;
+          break;
+        }
+      }
+    }
+    if (go && ld_relaxed_i32(&ctl->abort)) go = 0;
+    __threadfence();
+    s_xgo = go;
+  }
+  __syncthreads();
+  return s_xgo != 0;
 }
 
 // Exact reduction of the NV dot products accumulated in the CTAs' shared
@@ -260,8 +284,7 @@ __device__ __forceinline__ bool grid_reduce_exact(GridTeam& tm, double (&out)[NV
     if (threadIdx.x < kExactSlots) ctl->xbad[en][threadIdx.x] = 0u;
   }
   ++tm.xepoch;
-  const unsigned long long epoch = tm.epoch++;
-  if (!exact_barrier(ctl, epoch, red, tm.timeout_ns)) return false;
+  if (!exact_barrier(ctl, tm.xepoch, tm.timeout_ns)) return false;
   // the totals, read past L1 (other SMs' atomics landed in L2); the CTA's own
   // accumulators are zero again and serve as scratch
   for (int t = threadIdx.x; t < NV * kExactLimbs; t += blockDim.x)
