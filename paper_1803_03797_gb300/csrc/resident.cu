@@ -206,7 +206,7 @@ int resident_batched(int count, const int* nx, const int* ny, const int* ld, con
   // launch, larger ones a launch of the next size they fit on; the base with the
   // least total time.
   std::vector<int> sizes;
-  for (int n : {19, 16, 12, 8, 6, 4, 3, 2, 1}) sizes.push_back(std::max(1, sms / n));
+  for (int n : kTeamSplits) sizes.push_back(team_size(sms, n));
   auto classes = [&](int base) {
     std::vector<std::vector<ResPick>> c(sizes.size());
     for (const ResPick& p : picks) {
@@ -222,7 +222,7 @@ int resident_batched(int count, const int* nx, const int* ny, const int* ld, con
     const auto c = classes(base);
     double us = 0.0;
     for (size_t s = 0; s < c.size(); ++s)
-      if (!c[s].empty()) us += res_makespan(kind, c[s], nx, ny, sizes[s], sms / sizes[s], min_rows);
+      if (!c[s].empty()) us += res_makespan(kind, c[s], nx, ny, sizes[s], team_count(sms, sizes[s]), min_rows);
     if (base == 0 || us < best_us) {
       best = base;
       best_us = us;
@@ -231,13 +231,12 @@ int resident_batched(int count, const int* nx, const int* ny, const int* ld, con
   const auto c = classes(best);
   // message memory: the abort flag, per launch a queue head and a word a team, then
   // the instances'; all of it starts at zero
-  constexpr size_t kLaunchBytes = 256 + 32 * kSlotWords * 8;
   size_t off = first_off + kAlign;
   std::vector<size_t> launch_off(c.size(), 0);
   for (size_t s = 0; s < c.size(); ++s)
     if (!c[s].empty()) {
       launch_off[s] = off;
-      off += kLaunchBytes;
+      off += kTeamLaunchBytes;
     }
   std::vector<BatchEntry> tab;
   std::vector<int> first(c.size(), 0);
@@ -281,7 +280,7 @@ int resident_batched(int count, const int* nx, const int* ny, const int* ld, con
     l.tab = dtab + first[s];
     l.ws = ws;
     l.next = reinterpret_cast<unsigned*>(ws + launch_off[s]);
-    l.item = reinterpret_cast<u64*>(ws + launch_off[s] + 256);
+    l.item = reinterpret_cast<u64*>(ws + launch_off[s] + kTeamWordOffset);
     l.errs = errs;
     l.abort_flag = reinterpret_cast<int*>(ws + first_off);
     l.info = info;
@@ -296,7 +295,7 @@ int resident_batched(int count, const int* nx, const int* ny, const int* ld, con
     l.a.max_outer = o.max_outer > 0 ? o.max_outer : 60;
     l.a.maxit_inner = o.maxit_inner;
     l.a.tol_inner = o.tol_inner > 0.0 ? o.tol_inner : 1e-4;
-    const int teams = std::min(sms / sizes[s], n);
+    const int teams = std::min(team_count(sms, sizes[s]), n);
     rc = res_launch_batch(res_batch_kernel_of(kind), l, teams, smem[s], st);
     if (rc != LAP5CG_OK) return rc;
   }

@@ -2,6 +2,7 @@
 // single and batched, instantiated one solve kind a translation unit.
 #pragma once
 
+#include "batch_teams.h"
 #include "launch.h"
 #include "resident.cuh"
 
@@ -86,7 +87,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) k_resident_batch(const ResB
   __shared__ int s_item;
   extern __shared__ __align__(16) unsigned char dsm[];
   const int team = (int)blockIdx.x / l.team, rank = (int)blockIdx.x - team * l.team;
-  u64* word = l.item + (size_t)team * kSlotWords;
+  u64* word = l.item + (size_t)team * kTeamWordStride;
   uint32_t seq = 0;
   for (;;) {
     // The team's first CTA draws an item and passes it on.  A CTA that an
