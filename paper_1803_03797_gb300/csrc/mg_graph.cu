@@ -1237,7 +1237,11 @@ static int gm_build(const SolvePlan& p, const PcgArgs<TM>& a, bool use_mid, cuda
   if (rc != LAP5CG_OK) return rc;
   GmScal* sc = reinterpret_cast<GmScal*>(p.ws + 1024);
   GmBind* bd = reinterpret_cast<GmBind*>(p.ws + 2048);
-  double* part = reinterpret_cast<double*>(p.ws + 4096);
+  constexpr size_t kPartOffset = 4096;
+  static_assert(1024 + sizeof(GmScal) <= 2048 && 2048 + sizeof(GmBind) <= kPartOffset, "control block");
+  static_assert(kPartOffset + 4 * kGmMaxBlocks * sizeof(double) <= kMidFlagOffset, "two sets of partial sums");
+  static_assert(kMidFlagOffset + kMidFlagBytes <= kCtlBytes, "the flags");
+  double* part = reinterpret_cast<double*>(p.ws + kPartOffset);
   const int nx = p.nx, ny = p.ny;
   const void* f_pass = reinterpret_cast<const void*>(&k_gm_pass<TM>);
   const void* f_init = reinterpret_cast<const void*>(&k_gm_init<TM>);

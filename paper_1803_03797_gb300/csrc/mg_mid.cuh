@@ -34,7 +34,8 @@ constexpr int kMidThreads = 512;
 constexpr int kMidMaxCtas = 160;
 constexpr int kMidMaxLevels = 12;                 // distributed levels
 constexpr int kMidStages = 2 * kMidMaxLevels + 2; // flag rows: down, small, up
-constexpr size_t kMidFlagOffset = 128 * 1024;     // flags in the workspace's control block
+constexpr size_t kMidFlagOffset = 160 * 1024;     // flags in the workspace's control block
+constexpr size_t kMidFlagBytes = (size_t)(kMidStages * kMidMaxCtas + 1) * sizeof(int);  // and the abort flag
 // Levels of at most this many points run on the last CTA alone: below, a level's
 // passes between CTA barriers cost less than two exchanges (binary64: FP64 pipe time
 // of one SM, 4 us per 400 points and V-cycle).
