@@ -136,7 +136,8 @@ typedef struct {
                                (IR_F32: 4 (nx + ny) + 50; IR_BF16PR: 2 (nx + ny) + 50) */
   int32_t max_outer;        /* IR: refinement step cap; 0 = default (60) */
   double tol_inner;         /* IR: inner relative tolerance; <= 0 = default (1e-4 F32, 1e-2 BF16) */
-  double timeout_s;         /* device barrier time limit in seconds; <= 0 = default (2 s) */
+  double timeout_s;         /* time limit in seconds of a wait between CTAs (barriers, reductions,
+                               neighbour exchanges); <= 0 = default (2 s) */
   double* history;          /* optional device array of maxit+1 doubles: recursive
                                relative residual after each update; NULL = off
                                (single solves only) */

@@ -60,11 +60,12 @@ struct GmBind {
   double* history;
   double tol;
   int maxit, pad;
+  long long timeout_ns;  // limit of the middle levels' waits
 };
 
 __global__ void k_gm_bind(GmBind* bd, const double* b, double* x, lap5cg_info* info, double* history, double tol,
-                          int maxit) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) *bd = GmBind{b, x, info, history, tol, maxit, 0};
+                          int maxit, long long timeout_ns) {
+  if (threadIdx.x == 0 && blockIdx.x == 0) *bd = GmBind{b, x, info, history, tol, maxit, 0, timeout_ns};
 }
 
 enum { GP_JAC = 0, GP_JAC_DOT, GP_RES, GP_RESTRICT, GP_PROLONG, GP_RES_RESTRICT, GP_PROLONG_JAC, GP_JAC_RES_RESTRICT };
@@ -681,9 +682,10 @@ __global__ void __launch_bounds__(512) k_gm_small(const GmScal* sc, GmLevels<TM>
 // The levels from m.lv[0] on (mg_mid.cuh): m.n distributed ones, then
 // [small_first, nlev) on the last CTA.
 template <class TM>
-__global__ void __launch_bounds__(kMidThreads, 1) k_gm_mid(GmScal* sc, MidArgs<TM> m, GmLevels<TM> levels, int nlev,
-                                                           int small_first, int nu_c) {
+__global__ void __launch_bounds__(kMidThreads, 1) k_gm_mid(GmScal* sc, const GmBind* bd, MidArgs<TM> m,
+                                                           GmLevels<TM> levels, int nlev, int small_first, int nu_c) {
   if (sc->stop) return;
+  const long long limit = bd->timeout_ns;
   extern __shared__ __align__(16) unsigned char gsm[];
   TM* sm = reinterpret_cast<TM*>(gsm);
   const int cta = (int)blockIdx.x, tag = sc->iters + 1, n = m.n;
@@ -698,7 +700,7 @@ __global__ void __launch_bounds__(kMidThreads, 1) k_gm_mid(GmScal* sc, MidArgs<T
   // written; n + 1 the small levels' result; n + 1 + l the result of level n - l
   if (cta == (int)gridDim.x - 1) {
     for (int i = threadIdx.x; i < tiny_elems<TM>(levels.lv, small_first, nlev); i += blockDim.x) sm[i] = TM(0);
-    if (!mid_wait(flags(n), 0, m.lv[n - 1].G - 1, tag, m.abort_flag)) return fail();
+    if (!mid_wait(flags(n), 0, m.lv[n - 1].G - 1, tag, m.abort_flag, limit)) return fail();
     tiny_levels<TM>(levels.lv, small_first, nlev, nu_c, sm, levels.lv[small_first].u);
     mid_signal(flags(n + 1), tag);
     return;
@@ -712,7 +714,7 @@ __global__ void __launch_bounds__(kMidThreads, 1) k_gm_mid(GmScal* sc, MidArgs<T
     if (l > 0) {  // the owners of the centre rows of b rows s - 3 .. e + 2
       const MidLevel<TM>& F = m.lv[l - 1];
       const int j0 = 2 * max(s - 3, 0) + 1, j1 = 2 * min(e + 2, L.g.ny - 1) + 1;
-      if (!mid_wait(flags(l), j0 / F.R, j1 / F.R, tag, m.abort_flag)) return fail();
+      if (!mid_wait(flags(l), j0 / F.R, j1 / F.R, tag, m.abort_flag, limit)) return fail();
     }
     mid_down<TM>(L, below(l), sm, m.offT, cta);
     mid_signal(flags(l + 1) + cta, tag);
@@ -724,13 +726,13 @@ __global__ void __launch_bounds__(kMidThreads, 1) k_gm_mid(GmScal* sc, MidArgs<T
     const TM* eg;
     TM* E;
     if (l == n - 1) {
-      if (!mid_wait(flags(n + 1), 0, 0, tag, m.abort_flag)) return fail();
+      if (!mid_wait(flags(n + 1), 0, 0, tag, m.abort_flag, limit)) return fail();
       eg = levels.lv[small_first].u;
       E = sm + m.offE;
     } else {
       const MidLevel<TM>& C = m.lv[l + 1];
       const int J0 = max(((s - 2) >> 1) - 1, 0), J1 = min((e + 1) >> 1, C.g.ny - 1);
-      if (!mid_wait(flags(2 * n - l), J0 / C.R, J1 / C.R, tag, m.abort_flag)) return fail();
+      if (!mid_wait(flags(2 * n - l), J0 / C.R, J1 / C.R, tag, m.abort_flag, limit)) return fail();
       eg = C.g.u;
       E = sm + C.offB;  // that level is done: its rows take the correction
     }
@@ -1326,7 +1328,7 @@ static int gm_build(const SolvePlan& p, const PcgArgs<TM>& a, bool use_mid, cuda
         int nlev = a.nlev, nu_c = a.nu_c;
         mid.flags = flags;
         mid.abort_flag = flags + kMidStages * kMidMaxCtas;
-        void* args[] = {&sc, &mid, &lv, &nlev, &mid_small, &nu_c};
+        void* args[] = {&sc, &bd, &mid, &lv, &nlev, &mid_small, &nu_c};
         if ((rc = gm_add(body, &bp, fm, (unsigned)mid_grid, kMidThreads, args, (unsigned)mid_smem)) != LAP5CG_OK)
           return fail(rc);
         cudaLaunchAttributeValue coop = {};
@@ -1505,7 +1507,8 @@ int solve_mg_graph(const SolvePlan& p, const PcgArgs<TM>& a, cudaStream_t st, bo
     g_gm_cache.push_back({key, exec});
   }
   k_gm_bind<<<1, 32, 0, st>>>(reinterpret_cast<GmBind*>(p.ws + 2048), static_cast<const double*>(p.b),
-                              static_cast<double*>(p.x), p.info, p.opts.history, p.tol, p.maxit);
+                              static_cast<double*>(p.x), p.info, p.opts.history, p.tol, p.maxit,
+                              (long long)((p.opts.timeout_s > 0.0 ? p.opts.timeout_s : 2.0) * 1e9));
   if (cudaGetLastError() != cudaSuccess || cudaGraphLaunch(exec, st) != cudaSuccess) return LAP5CG_ERR_CUDA;
   *used = true;
   return LAP5CG_OK;

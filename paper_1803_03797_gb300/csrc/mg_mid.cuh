@@ -21,7 +21,7 @@
 // no rows; it runs the levels below the distributed ones on its own.
 //
 // Flags count V-cycles (zeroed at the start of a solve, so no value repeats);
-// every wait is bounded (2 s), after which the solve ends with
+// every wait is bounded (opts.timeout_s), after which the solve ends with
 // LAP5CG_ERR_SYNC_TIMEOUT.  The launch is cooperative: the CTAs wait for one another.
 #pragma once
 
@@ -146,7 +146,8 @@ __device__ __forceinline__ void mid_store(TM* p, int x, int nx, bool live, TM (&
 
 // Waits for flags [c0, c1] of a stage to reach tag.  False (in every thread) when
 // the solve must stop.
-__device__ __forceinline__ bool mid_wait(const int* flags, int c0, int c1, int tag, int* abort_flag) {
+__device__ __forceinline__ bool mid_wait(const int* flags, int c0, int c1, int tag, int* abort_flag,
+                                         long long timeout_ns) {
   bool fail = false;
   for (int c = c0 + (int)threadIdx.x; c <= c1 && !fail; c += blockDim.x) {
     unsigned spins = 0;
@@ -154,7 +155,7 @@ __device__ __forceinline__ bool mid_wait(const int* flags, int c0, int c1, int t
     while (ld_relaxed_i32(flags + c) != tag) {
       const unsigned long long now = global_ns();
       if (spins++ == 0u) t0 = now;
-      if (((spins & 31u) == 0u && ld_relaxed_i32(abort_flag)) || now - t0 > 2000000000ull) {
+      if (((spins & 31u) == 0u && ld_relaxed_i32(abort_flag)) || (long long)(now - t0) > timeout_ns) {
         atomicExch(abort_flag, 1);
         fail = true;
         break;

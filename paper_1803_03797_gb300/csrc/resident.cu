@@ -287,6 +287,7 @@ int resident_batched(int count, const int* nx, const int* ny, const int* ld, con
     l.count = n;
     l.team = sizes[s];
     l.min_rows = min_rows;
+    l.timeout_ns = (long long)((o.timeout_s > 0.0 ? o.timeout_s : 2.0) * 1e9);
     l.a = ResArgs();
     l.a.history = nullptr;
     l.a.tol = tol;

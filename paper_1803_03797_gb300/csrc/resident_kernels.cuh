@@ -70,6 +70,7 @@ struct ResBatchLaunch {
   int *errs, *abort_flag;
   lap5cg_info* info;
   int count, team, min_rows;
+  long long timeout_ns;
   ResArgs a;              // what all instances share
 };
 
@@ -138,7 +139,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) k_resident_batch(const ResB
       u64* mem = reinterpret_cast<u64*>(l.ws + e.ws_off);
       ResTeam tm;
       tm.init(mem, mem + (size_t)2 * ctas * kSlotWords, rank, ctas, groups, l.errs + e.idx, l.abort_flag,
-              2000000000LL, &sh);
+              l.timeout_ns, &sh);
       res_body_of<KIND>((rows * groups + kResMaxThreads - 1) / kResMaxThreads, a, tm, reinterpret_cast<T*>(dsm));
     }
     __syncthreads();  // the shared rows and scalars are the next instance's
