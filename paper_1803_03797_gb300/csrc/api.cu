@@ -48,11 +48,17 @@ int warps_of(const lap5cg_opts& o) {
 
 static int ring_warp_bytes(int S, int slot_bytes) { return (int)align_up(128 + (size_t)S * slot_bytes, 128); }
 
-lap5cg_opts with_warps(const lap5cg_opts& o, int slot_bytes) {
+lap5cg_opts with_warps(const lap5cg_opts& o, int slot_bytes, int nx, int ny, int V) {
   lap5cg_opts r = o;
   r.warps_per_cta = warps_of(o);
   DevProps dp;
-  if (o.warps_per_cta > 0 || o.ring_slots <= 0 || dev_props(&dp) != LAP5CG_OK) return r;
+  if (o.warps_per_cta > 0 || dev_props(&dp) != LAP5CG_OK) return r;
+  if (o.ctas <= 0) {
+    const Units un = make_units(nx, ny, V, (long long)dp.sms * r.warps_per_cta, o.min_rows > 0 ? o.min_rows : kDefaultMinRows);
+    const int need = (int)((un.nunits + dp.sms - 1) / dp.sms);
+    if (need < r.warps_per_cta) r.warps_per_cta = need > kPollWarps ? need : kPollWarps;
+  }
+  if (o.ring_slots <= 0) return r;
   const int S = o.ring_slots < 3 ? 3 : (o.ring_slots > kRingMaxSlots ? kRingMaxSlots : o.ring_slots);
   while (r.warps_per_cta > 4 &&
          (size_t)r.warps_per_cta * ring_warp_bytes(S, slot_bytes) + 4096 > (size_t)dp.max_smem_optin)

@@ -117,7 +117,8 @@ int solve_typed(const SolvePlan& plan, cudaStream_t st) {
   SolvePlan p = plan;
   if (EX && p.opts.warps_per_cta == 0) p.opts.warps_per_cta = kExactWarps;
   p.opts = with_warps(p.opts, plan.variant == LAP5CG_CLASSIC ? ring_slot_classic(V, (int)sizeof(T))
-                                                                : ring_slot_newcg(V, (int)sizeof(T)));
+                                                                : ring_slot_newcg(V, (int)sizeof(T)),
+                      p.nx, p.ny, V);
   const size_t vec = align_up((size_t)p.ny * (size_t)p.ldw * sizeof(T), kAlign);
   unsigned char* base = p.ws + kCtlBytes;
   auto vecp = [&](int k) { return reinterpret_cast<T*>(base + (size_t)k * vec); };

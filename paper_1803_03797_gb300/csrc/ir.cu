@@ -36,7 +36,7 @@ size_t ws_bytes_ir(int nx, int ny, int variant, int precision) {
 template <class TR, int V>
 static int solve_ir_t(const SolvePlan& plan, cudaStream_t st) {
   SolvePlan p = plan;
-  p.opts = with_warps(plan.opts, ring_slot_ir(V, (int)sizeof(TR)));
+  p.opts = with_warps(plan.opts, ring_slot_ir(V, (int)sizeof(TR)), p.nx, p.ny, V);
   const int ldi = inner_ld(p.nx);
   const size_t vr = align_up((size_t)p.ny * ldi * sizeof(TR), kAlign);
   const size_t vf = align_up((size_t)p.ny * ldi * 4, kAlign);

@@ -120,9 +120,13 @@ int choose_ring(const void* func, int slot_bytes, const lap5cg_opts& o, int wpc,
 
 // Warps per CTA of the single-grid kernels for these options.
 int warps_of(const lap5cg_opts& o);
-// The options with warps_per_cta filled in for a kernel with ring slots of
-// slot_bytes: the default, or fewer where an explicit ring_slots would not fit.
-lap5cg_opts with_warps(const lap5cg_opts& o, int slot_bytes);
+// The options with warps_per_cta filled in for a kernel of V columns a lane with ring
+// slots of slot_bytes: the default; fewer where an explicit ring_slots would not fit,
+// and on grids with fewer units than the SMs hold warps, which are then spread over the
+// SMs (kPollWarps at least: the reductions' messages need them).  Us an iteration with 16
+// warps, on 2 to 50 SMs, and so: NewCG with residual replacement 64^2 15.1 and 9.9, 300^2
+// 15.7 and 10.9; classic 64^2 12.8 and 9.8; the spare FP64 pipes are what it gains.
+lap5cg_opts with_warps(const lap5cg_opts& o, int slot_bytes, int nx, int ny, int V);
 
 // Largest ring slot (bytes) of each kernel family, V = lane vector width.
 inline int ring_slot_classic(int V, int es) {
