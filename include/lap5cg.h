@@ -80,7 +80,11 @@ typedef enum { LAP5CG_DT_F64 = 0, LAP5CG_DT_F32 = 1, LAP5CG_DT_BF16 = 2 } lap5cg
 typedef enum { LAP5CG_CLASSIC = 0, LAP5CG_NEWCG = 1 } lap5cg_variant;
 
 /* Precision of a solve.
- *   F64      : b, x binary64; all arithmetic binary64.
+ *   F64      : b, x binary64; all arithmetic binary64.  A p may be summed in
+ *              64-bit fixed point where its error bound at every point (24 to
+ *              29 x 2^-53 of the point's largest operand) is that of the four
+ *              binary64 operations (26 x 2^-53); elsewhere, and always in the
+ *              reproducible mode and lap5_apply, in binary64.
  *   F32      : b, x binary32; arithmetic binary32, dot products accumulated
  *              with compensated (Dot2) summation, scalars in binary64.
  *   IR_F32   : b, x binary64.  Outer FP64 iterative refinement (residual
@@ -149,7 +153,8 @@ typedef struct {
                                row. */
   int32_t ring_slots;       /* rows each warp keeps in flight in its shared-memory ring
                                (bulk asynchronous copies): 0 = automatic (on when the warp
-                               units are at least 8 rows tall),
+                               units are at least 8 rows tall; 5 where the library chose
+                               wide lanes: eight binary32 or four binary64 columns),
                                3..8 = that many, < 0 = no ring (rows loaded into registers) */
   int32_t resident;         /* 0 (default): F64, F32 classic and IR_F32 solves whose vectors fit in
                                the registers and shared memory of the chip (about 1060^2
@@ -163,9 +168,9 @@ typedef struct {
   int32_t lane_vec;         /* columns each lane owns in its warp's strip.
                                Binary32 passes (F32 classic; the inner passes of IR_F32 /
                                IR_BF16PR): 4 or 8; 0 = automatic (8 when nx >= 1024 and the
-                               ring is used).  8 needs the classic variant and the
-                               shared-memory ring (ring_slots > 0, or automatic with units at
-                               least 8 rows tall), and store_z <= 0 for IR.
+                               warp units are at least 5 rows tall).  8 needs the classic
+                               variant and the shared-memory ring (ring_slots > 0, or automatic
+                               with units at least 8 rows tall), and store_z <= 0 for IR.
                                F64: 2 or 4; 0 = automatic (4 for classic CG with the ring when
                                ld is a multiple of 4, else 2).  4 needs the classic variant,
                                the ring and ld a multiple of 4; the reproducible mode takes 2.

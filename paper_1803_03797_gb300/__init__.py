@@ -276,8 +276,8 @@ def batched_workspace_size(nx_list, ny_list, ld_list, variant="classic", precisi
 
 def cg_solve_batched(bs, xs=None, tol=1e-10, maxit=100000, variant="classic", precision="ir_f32", nx_list=None,
                      opts: Opts = None, workspace=None, info=None, stream=None):
-    """Solve len(bs) independent systems of different shapes in one persistent
-    launch.  bs: list of (ny, ld) CUDA tensors.  Returns (xs, info)."""
+    """Solve len(bs) independent systems of different shapes in one call (a few
+    persistent launches).  bs: list of (ny, ld) CUDA tensors.  Returns (xs, info)."""
     n = len(bs)
     if n < 1:
         raise ValueError("empty batch")

@@ -1,9 +1,10 @@
 // batched.cu -- cg_solve_batched: many independent grids of different shapes
-// in one persistent launch.
+// in one call, a few persistent launches.
 //
 // Instances whose state fits in the SMs of a team go to the chip-resident
-// kernels first (resident.cu; a launch or a few for all of them); what follows
-// is for the rest.  A team is one thread-block cluster (1, 2, 4, 8 or 16 CTAs).  Teams pull the
+// kernels first (resident.cu; one launch a team size), then those that fit in one
+// cluster's shared memory to small.cu; what follows is for the rest, one
+// launch.  A team is one thread-block cluster (1, 2, 4, 8 or 16 CTAs).  Teams pull the
 // next instance from an atomic queue over a table sorted by estimated work
 // (largest first: grid points x (nx + ny), since CG iterations grow with the
 // side length), solve it with the same fused passes as the single-grid

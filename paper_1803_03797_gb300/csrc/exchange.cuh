@@ -5,6 +5,8 @@
 //  * Messages carry their own flags.  A value travels as 64-bit words of 32 data
 //    and 32 tag bits (relaxed 64-bit accesses are single-copy atomic), so a
 //    receiver polls the data itself: no fence, no separate flag, one L2 round trip.
+//    (The idea is that of NCCL's low-latency (LL) protocol: 8-byte stores of 4 bytes of
+//    data and a 4-byte flag.)
 //    An exchange of one value among 152 CTAs, one 256-byte slot a CTA polled by one
 //    lane each, measured 1.1 us (1.6 us with five slots a lane; 4.1 us with 16-byte
 //    slots, whose lines writers and pollers share; 1.9 us with an inbox a CTA).

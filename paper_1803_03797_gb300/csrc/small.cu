@@ -2,8 +2,8 @@
 // whole grid lives in the shared memory of one thread-block cluster of up to
 // 16 CTAs.  By default resident.cu takes these grids first (faster from 100^2
 // on: NewCG 3.8 against 6.2 us an iteration, classic 4.7 against 6.5); this
-// kernel runs for an explicit team_ctas and where the messages of resident.cu
-// have no room in the workspace.
+// kernel runs for an explicit team_ctas, for binary32 NewCG, and where the messages
+// of resident.cu have no room in the workspace.
 //
 // CTA c of the cluster owns a contiguous block of rows of every state vector
 // in its shared memory, with one halo row above and below.  After a stencil
